@@ -1088,10 +1088,28 @@ int hhg_create_mesh(const double* V, int64_t nv, const int32_t* T, int64_t nt, c
       M->err = cerr;
       return bail(HHG_EMESH);
     }
+    // the rows of A side by side (CoarseSys::ecol)
+    const int32_t arows = (int32_t)cm.aptr.size() - 1;
+    std::vector<double> eval;
+    std::vector<int32_t> ecol;
+    if (arows > 0 && arows <= COARSE_ELL_MAX_ROWS) {
+      int32_t width = 1;
+      for (int32_t r = 0; r < arows; ++r) width = std::max(width, cm.aptr[r + 1] - cm.aptr[r]);
+      width = (width + COARSE_ELL_ROUND - 1) / COARSE_ELL_ROUND * COARSE_ELL_ROUND;
+      eval.assign((size_t)width * arows, 0.0);
+      ecol.resize((size_t)width * arows);
+      for (int32_t r = 0; r < arows; ++r)
+        for (int32_t e = 0; e < width; ++e) {
+          const int32_t k = cm.aptr[r] + e;
+          const bool have = k < cm.aptr[r + 1];
+          ecol[(size_t)e * arows + r] = have ? cm.acol[k] : r;
+          if (have) eval[(size_t)e * arows + r] = cm.aval[k];
+        }
+    }
     // one allocation, 8-byte aligned parts: doubles first, then the indices
-    const size_t nd = cm.kval.size() + cm.aval.size() + cm.mass.size();
+    const size_t nd = cm.kval.size() + cm.aval.size() + cm.mass.size() + eval.size();
     const size_t ni = cm.vidx.size() + cm.pidx.size() + cm.kptr.size() + cm.kcol.size() + cm.aptr.size() +
-                      cm.acol.size();
+                      cm.acol.size() + ecol.size();
     if ((rc = dalloc(M, &M->d_coarse_sys, sizeof(double) * nd + sizeof(int32_t) * ni + 16))) return bail(rc);
     double* dp = (double*)M->d_coarse_sys;
     int32_t* ip = (int32_t*)(dp + nd);
@@ -1114,12 +1132,14 @@ int hhg_create_mesh(const double* V, int64_t nv, const int32_t* T, int64_t nt, c
     S.kval = put_d(cm.kval);
     S.aval = put_d(cm.aval);
     S.mass = put_d(cm.mass);
+    S.eval = eval.empty() ? nullptr : put_d(eval);
     S.vidx = put_i(cm.vidx);
     S.pidx = put_i(cm.pidx);
     S.kptr = put_i(cm.kptr);
     S.kcol = put_i(cm.kcol);
     S.aptr = put_i(cm.aptr);
     S.acol = put_i(cm.acol);
+    S.ecol = ecol.empty() ? nullptr : put_i(ecol);
     if ((e = cudaGetLastError()) != cudaSuccess) {
       M->err = std::string("upload of the coarse system: ") + cudaGetErrorString(e);
       return bail(HHG_ECUDA);

@@ -34,14 +34,16 @@ __device__ __forceinline__ double csr_row(const int32_t* ptr, const int32_t* col
                                           const double* x) {
   double s = 0.0;
   const int e = ptr[r + 1];
+#pragma unroll 4
   for (int k = ptr[r]; k < e; ++k) s += val[k] * x[col[k]];
   return s;
 }
 
-__device__ inline double dot(const Ctx& C, const double* a, const double* b) {
+// This thread's part of a.b.
+__device__ __forceinline__ double dot_part(const Ctx& C, const double* a, const double* b) {
   double s = 0;
   for (int q = (int)C.T.rank(); q < C.n; q += (int)C.T.size()) s += a[q] * b[q];
-  return team_sum1(C.T, s);
+  return s;
 }
 
 // y = K x
@@ -50,144 +52,282 @@ __device__ inline void applyK(const Ctx& C, const double* x, double* y) {
   C.T.sync();
 }
 
-// x_d = CG(A, b_d) from zero for the three velocity blocks in lockstep over
-// the team: each block follows the stopping rule of the single CG on its own
-// (it stops before an iteration when r.r <= rtol^2 r0.r0 or r.r = 0, or when
-// d.Ad = 0), the others go on; sums of the three blocks share one team
-// reduction.  b, x: 3 nv entries; cg: 9 nv scratch (r, d, A d per block).
-// Returns the iterations summed over the blocks.
-__device__ inline int cg3(const Ctx& C, const double* b, double* x, double* cg, int max_it, double rtol) {
-  const int nv = C.S.nv;
-  double* R = cg;
-  double* D = cg + 3 * nv;
-  double* Q = cg + 6 * nv;
-  for (int q = (int)C.T.rank(); q < 3 * nv; q += (int)C.T.size()) {
-    x[q] = 0.0;
-    R[q] = b[q];
-    D[q] = b[q];
-    Q[q] = 0.0;
-  }
-  C.T.sync();
-  double rr[3] = {0, 0, 0};
-  for (int q = (int)C.T.rank(); q < nv; q += (int)C.T.size())
+// ---- team CG -----------------------------------------------------------------
+// x_s = CG(A, b_s) from zero for NSYS systems in lockstep over the team: the
+// three velocity components with the scalar A (NSYS = 3, N = nv rows each) or
+// the coupled block of the D form and of free slip (NSYS = 1, N = 3 nv rows).
+// Each system follows the stopping rule of a single CG on its own (it stops
+// before an iteration when r.r <= rtol^2 r0.r0 or r.r = 0, or when d.Ad = 0);
+// the others go on.  b, x: NSYS N entries.  Returns the iterations summed
+// over the systems.
+//
+// cg_team_regs: a CTA holds a run of rows of every system and a thread at
+// most one (system, row) pair, whose x, r, d, A d and first CG_ROW matrix
+// entries (with the addresses of their directions) stay in registers; a
+// warp's pairs belong to one system.  The directions lie in the shared memory
+// of their CTAs, dir, and are read through the cluster's shared window.  An
+// iteration is three cluster barriers: d.Ad, r.r and the new directions.  It
+// is bound by the latencies of the FP64 chain (64 cycles per dependent
+// operation, 560 per division) and of the barriers (480 cycles each).
+constexpr int CG_ROW = COARSE_ELL_ROUND;
+constexpr int CG_DIR = 512;  // directions of a CTA: one per thread
+
+template <int NSYS>
+__device__ __noinline__ int cg_team_regs(const Ctx& C, const double* b, double* x, double* dir, int max_it,
+                                         double rtol) {
+  const int N = NSYS == 3 ? C.S.nv : 3 * C.S.nv;
+  const int rc = (N + (int)C.T.nblocks - 1) / (int)C.T.nblocks;  // rows per CTA
+  const int rp = (rc + 31) / 32 * 32;                            // padded: whole warps per system
+  const int each = rp / 32;                                      // warps per system
+  const int sys = (int)(threadIdx.x >> 5) / each;
+  const bool used = sys < NSYS;
+  const int l = (int)threadIdx.x - sys * rp;  // row within the CTA
+  const int row = (int)blockIdx.x * rc + l;
+  const bool on = used && l < rc && row < N;
+  const int idx = on ? sys * N + row : -1;
+  const int mine = used ? sys : 0;
+  const uint32_t dir0 = (uint32_t)__cvta_generic_to_shared(dir) + 8u * (uint32_t)(mine * rp);
+  const uint32_t inv = 0xffffffffu / (uint32_t)rc + 1u;  // col / rc = umulhi(col, inv): col, rc < 2^13 (rc = 1: inv = 0)
+  auto addr_of = [&](int col) {
+    const uint32_t o = rc == 1 ? (uint32_t)col : __umulhi((uint32_t)col, inv);
+    const uint32_t at = dir0 + 8u * ((uint32_t)col - o * (uint32_t)rc);
+    return C.T.nblocks > 1 ? team_shared_addr(at, o) : at;
+  };
+  // entries of the warp's longest row (the others' absent ones are zeros on
+  // their own directions; a thread without a row reads row 0 and drops it)
+  const int len = __reduce_max_sync(0xffffffffu, on ? C.S.aptr[row + 1] - C.S.aptr[row] : 0);
+  const double* ev = C.S.eval + (on ? row : 0);
+  const int32_t* ec = C.S.ecol + (on ? row : 0);
+  double av[CG_ROW];
+  uint32_t ad[CG_ROW];
 #pragma unroll
-    for (int d = 0; d < 3; ++d) rr[d] += R[d * nv + q] * R[d * nv + q];
-  team_sum<3>(C.T, rr);
-  double stop[3];
-  bool run[3];
-  for (int d = 0; d < 3; ++d) {
-    stop[d] = rtol * rtol * rr[d];
-    run[d] = true;
+  for (int e = 0; e < CG_ROW; ++e) {
+    av[e] = ev[(int64_t)e * N];
+    ad[e] = addr_of(ec[(int64_t)e * N]);
   }
+  double xv = 0.0, qv = 0.0, rv = on ? b[idx] : 0.0, dv = rv;
+  if (used) dir[mine * rp + l] = dv;
+  // state of the handler warps: r.r, the stopping bound, running, iterations
+  double rr = 0.0, stop = 0.0, inv_rr = 0.0;
+  bool run = false;
   int its = 0;
+  const double* res = team_reduce<NSYS, 2>(C.T, rv * rv, each, [&](int, double tot, double* out) {
+    rr = tot;
+    stop = rtol * rtol * tot;
+    run = !(rr <= stop || rr == 0.0);
+    out[0] = run ? 1.0 : 0.0;
+    out[1] = 0.0;
+  });
   for (int it = 0; it < max_it; ++it) {
-    for (int d = 0; d < 3; ++d)
-      if (rr[d] <= stop[d] || rr[d] == 0.0) run[d] = false;
-    if (!(run[0] || run[1] || run[2])) break;
-    for (int q = (int)C.T.rank(); q < nv; q += (int)C.T.size())
+    // the directions are published: by the sum above (first iteration) or the barrier below
+    bool any = false;
 #pragma unroll
-      for (int d = 0; d < 3; ++d)
-        if (run[d]) Q[d * nv + q] = csr_row(C.S.aptr, C.S.acol, C.S.aval, q, D + d * nv);
-    C.T.sync();
-    double dq[3] = {0, 0, 0};
-    for (int q = (int)C.T.rank(); q < nv; q += (int)C.T.size())
+    for (int s = 0; s < NSYS; ++s) any |= res[2 * s] != 0.0;
+    if (!any) break;
+    bool go = used && res[2 * mine] != 0.0;
+    double acc = 0.0;
+    if (go) {
+      double dn[CG_ROW];
 #pragma unroll
-      for (int d = 0; d < 3; ++d)
-        if (run[d]) dq[d] += D[d * nv + q] * Q[d * nv + q];
-    team_sum<3>(C.T, dq);
-    double alpha[3];
-    for (int d = 0; d < 3; ++d) {
-      if (run[d] && dq[d] == 0.0) run[d] = false;
-      alpha[d] = run[d] ? rr[d] / dq[d] : 0.0;
-    }
-    double rn[3] = {0, 0, 0};
-    for (int q = (int)C.T.rank(); q < nv; q += (int)C.T.size())
+      for (int e = 0; e < CG_ROW; ++e) dn[e] = ld_team_shared(ad[e]);
+      qv = 0.0;
 #pragma unroll
-      for (int d = 0; d < 3; ++d)
-        if (run[d]) {
-          const int i = d * nv + q;
-          x[i] += alpha[d] * D[i];
-          R[i] -= alpha[d] * Q[i];
-          rn[d] += R[i] * R[i];
+      for (int e = 0; e < CG_ROW; ++e) qv += av[e] * dn[e];
+      for (int k = CG_ROW; k < len; k += CG_ROW) {
+        double a[CG_ROW];
+        uint32_t at[CG_ROW];
+#pragma unroll
+        for (int e = 0; e < CG_ROW; ++e) {
+          a[e] = __ldg(ev + (int64_t)(k + e) * N);
+          at[e] = addr_of(__ldg(ec + (int64_t)(k + e) * N));
         }
-    team_sum<3>(C.T, rn);
-    double beta[3];
-    for (int d = 0; d < 3; ++d) beta[d] = run[d] ? rn[d] / rr[d] : 0.0;
-    for (int q = (int)C.T.rank(); q < nv; q += (int)C.T.size())
 #pragma unroll
-      for (int d = 0; d < 3; ++d)
-        if (run[d]) D[d * nv + q] = R[d * nv + q] + beta[d] * D[d * nv + q];
-    C.T.sync();
-    for (int d = 0; d < 3; ++d)
-      if (run[d]) {
-        rr[d] = rn[d];
-        ++its;
+        for (int e = 0; e < CG_ROW; ++e) dn[e] = ld_team_shared(at[e]);
+#pragma unroll
+        for (int e = 0; e < CG_ROW; ++e)
+          if (k + e < len) qv += a[e] * dn[e];
       }
+      if (!on) qv = 0.0;
+      acc = dv * qv;
+    }
+    res = team_reduce<NSYS, 2>(C.T, acc, each, [&](int, double tot, double* out) {
+      double alpha;
+      div_and_rcp(rr, tot, rr, alpha, inv_rr);
+      if (run && tot == 0.0) run = false;
+      out[0] = run ? 1.0 : 0.0;
+      out[1] = run ? alpha : 0.0;
+    });
+    go = go && res[2 * mine] != 0.0;
+    acc = 0.0;
+    if (go) {
+      const double alpha = res[2 * mine + 1];
+      rv -= alpha * qv;
+      acc = rv * rv;
+      xv += alpha * dv;
+    }
+    res = team_reduce<NSYS, 2>(C.T, acc, each, [&](int, double tot, double* out) {
+      out[0] = out[1] = 0.0;
+      if (run) {
+        out[1] = tot * inv_rr;
+        rr = tot;
+        ++its;
+        run = !(rr <= stop || rr == 0.0);
+        out[0] = run ? 1.0 : 0.0;
+      }
+    });
+    if (go) {
+      dv = rv + res[2 * mine + 1] * dv;
+      dir[mine * rp + l] = dv;
+    }
+    C.T.sync();
   }
-  return its;
+  if (on) x[idx] = xv;
+  res = team_reduce<NSYS, 1>(C.T, 0.0, each, [&](int, double, double* out) { out[0] = (double)its; });
+  double n = 0.0;
+#pragma unroll
+  for (int s = 0; s < NSYS; ++s) n += res[s];
+  return (int)n;
 }
 
-// x = CG(A, b) from zero on the coupled D-form velocity block (3 nv rows of
-// A in CSR) over the team, same stopping rule; cg: 9 nv scratch.
-__device__ inline int cg_coupled(const Ctx& C, const double* b, double* x, double* cg, int max_it, double rtol) {
-  const int n = 3 * C.S.nv;
+// The same for any number of rows per thread, on vectors in global memory
+// (cg: r, d and A d, NSYS N entries each).
+template <int NSYS>
+__device__ __noinline__ int cg_team_mem(const Ctx& C, const double* b, double* x, double* cg, int max_it,
+                                        double rtol) {
+  const int N = NSYS == 3 ? C.S.nv : 3 * C.S.nv;
+  // the warps of a CTA in NSYS groups
+  const int each = (int)(blockDim.x >> 5) / NSYS;
+  const int warp = threadIdx.x >> 5, mine = min(warp / each, NSYS - 1);
+  // (a remainder warp has no rows)
+  const int t0 = warp < NSYS * each
+                     ? ((warp - mine * each) * (int)C.T.nblocks + (int)blockIdx.x) * 32 + (int)(threadIdx.x & 31)
+                     : N;
+  const int step = each * (int)C.T.nblocks * 32;
   double* R = cg;
-  double* D = cg + n;
-  double* Q = cg + 2 * n;
-  double rr = 0.0;
-  for (int q = (int)C.T.rank(); q < n; q += (int)C.T.size()) {
+  double* D = cg + NSYS * N;
+  double* Q = cg + 2 * NSYS * N;
+  b += mine * N;
+  x += mine * N;
+  R += mine * N;
+  D += mine * N;
+  Q += mine * N;
+  double acc = 0.0;
+  for (int q = t0; q < N; q += step) {
+    const double v = b[q];
     x[q] = 0.0;
-    R[q] = b[q];
-    D[q] = b[q];
-    rr += b[q] * b[q];
+    R[q] = v;
+    D[q] = v;
+    acc += v * v;
   }
-  rr = team_sum1(C.T, rr);
-  const double stop = rtol * rtol * rr;
-  int it = 0;
-  for (; it < max_it; ++it) {
-    if (rr <= stop || rr == 0.0) break;
-    double dq = 0.0;
-    for (int q = (int)C.T.rank(); q < n; q += (int)C.T.size()) {
-      const double aq = csr_row(C.S.aptr, C.S.acol, C.S.aval, q, D);
-      Q[q] = aq;
-      dq += D[q] * aq;
+  double rr = 0.0, stop = 0.0, inv_rr = 0.0;
+  bool run = false;
+  int its = 0;
+  const double* res = team_reduce<NSYS, 2>(C.T, acc, each, [&](int, double tot, double* out) {
+    rr = tot;
+    stop = rtol * rtol * tot;
+    run = !(rr <= stop || rr == 0.0);
+    out[0] = run ? 1.0 : 0.0;
+    out[1] = 0.0;
+  });
+  for (int it = 0; it < max_it; ++it) {
+    bool any = false;
+#pragma unroll
+    for (int s = 0; s < NSYS; ++s) any |= res[2 * s] != 0.0;
+    if (!any) break;
+    const bool on = res[2 * mine] != 0.0;
+    acc = 0.0;
+    if (on)
+      for (int q = t0; q < N; q += step) {
+        const double aq = csr_row(C.S.aptr, C.S.acol, C.S.aval, q, D);
+        Q[q] = aq;
+        acc += D[q] * aq;
+      }
+    res = team_reduce<NSYS, 2>(C.T, acc, each, [&](int, double tot, double* out) {
+      double alpha;
+      div_and_rcp(rr, tot, rr, alpha, inv_rr);
+      if (run && tot == 0.0) run = false;
+      out[0] = run ? 1.0 : 0.0;
+      out[1] = run ? alpha : 0.0;
+    });
+    const bool go = on && res[2 * mine] != 0.0;
+    const double alpha = res[2 * mine + 1];
+    acc = 0.0;
+    if (go)
+      for (int q = t0; q < N; q += step) {
+        x[q] += alpha * D[q];
+        const double rq = R[q] - alpha * Q[q];
+        R[q] = rq;
+        acc += rq * rq;
+      }
+    res = team_reduce<NSYS, 2>(C.T, acc, each, [&](int, double tot, double* out) {
+      out[0] = out[1] = 0.0;
+      if (run) {
+        out[1] = tot * inv_rr;
+        rr = tot;
+        ++its;
+        run = !(rr <= stop || rr == 0.0);
+        out[0] = run ? 1.0 : 0.0;
+      }
+    });
+    if (go) {
+      const double beta = res[2 * mine + 1];
+      for (int q = t0; q < N; q += step) D[q] = R[q] + beta * D[q];
     }
-    dq = team_sum1(C.T, dq);
-    if (dq == 0.0) break;
-    const double alpha = rr / dq;
-    double rn = 0.0;
-    for (int q = (int)C.T.rank(); q < n; q += (int)C.T.size()) {
-      x[q] += alpha * D[q];
-      R[q] -= alpha * Q[q];
-      rn += R[q] * R[q];
-    }
-    rn = team_sum1(C.T, rn);
-    const double beta = rn / rr;
-    for (int q = (int)C.T.rank(); q < n; q += (int)C.T.size()) D[q] = R[q] + beta * D[q];
     C.T.sync();
-    rr = rn;
   }
-  return it;
+  res = team_reduce<NSYS, 1>(C.T, 0.0, 0, [&](int, double, double* out) { out[0] = (double)its; });
+  double n = 0.0;
+#pragma unroll
+  for (int s = 0; s < NSYS; ++s) n += res[s];
+  return (int)n;
+}
+
+// Team CG of the preconditioner; cg: 9 nv entries of global scratch, dir:
+// CG_DIR entries of shared memory.  One row per thread covers nv <= 2,560 on
+// 16 CTAs of 512 threads.
+template <int NSYS>
+__device__ inline int cg_team(const Ctx& C, const double* b, double* x, double* cg, double* dir, int max_it,
+                              double rtol) {
+  const int N = NSYS == 3 ? C.S.nv : 3 * C.S.nv;
+  const int rc = (N + (int)C.T.nblocks - 1) / (int)C.T.nblocks;
+  if (C.S.eval && NSYS * ((rc + 31) / 32 * 32) <= min((int)blockDim.x, CG_DIR))
+    return cg_team_regs<NSYS>(C, b, x, dir, max_it, rtol);
+  return cg_team_mem<NSYS>(C, b, x, cg, max_it, rtol);
 }
 
 // ---- warp-level CG: the three velocity blocks are solved concurrently ------
 
-// Sum over the warp, the same value in every lane (shuffle tree, lane 0 broadcast).
-__device__ __forceinline__ double warp_sum(double v) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  return __shfl_sync(0xffffffffu, v, 0);
-}
-
-// x = CG(A, b) from zero by one warp (same stopping rule as cg3).
-__device__ inline int cg_warp(const CoarseSys& S, const double* b, double* x, double* r, double* d, double* w,
-                              int max_it, double rtol) {
+// x = CG(A, b) from zero by one warp (the same stopping rule), up to NR rows
+// per lane with x, r, d, A d and the first CG_ROW entries of each row in
+// registers; dir: the search direction in shared memory, nv entries of this
+// warp.  One lane per row and a butterfly per sum; an iteration of the cube's
+// level 2 (27 rows) is a chain of 7 row products, two trees of 5 additions
+// and two divisions in FP64, 64 cycles per operation and 560 per division.
+template <int NR>
+__device__ __noinline__ int cg_warp(const CoarseSys& S, const double* b, double* x, double* dir, int max_it, double rtol) {
   const int lane = threadIdx.x & 31, nv = S.nv;
+  constexpr bool KEEP = NR == 1;
+  double xv[NR], rv[NR], dv[NR], qv[NR], av[CG_ROW];
+  int at[NR], len[NR], ac[CG_ROW];  // a lane without a row reads row 0 and drops it
   double rr = 0.0;
-  for (int q = lane; q < nv; q += 32) {
-    x[q] = 0.0;
-    r[q] = b[q];
-    d[q] = b[q];
-    rr += b[q] * b[q];
+#pragma unroll
+  for (int m = 0; m < NR; ++m) {
+    const int q = lane + 32 * m;
+    const bool on = q < nv;
+    at[m] = on ? q : 0;
+    len[m] = __reduce_max_sync(0xffffffffu, on ? S.aptr[q + 1] - S.aptr[q] : 0);
+    if (KEEP) {
+#pragma unroll
+      for (int e = 0; e < CG_ROW; ++e) {
+        av[e] = S.eval[e * nv + at[m]];
+        ac[e] = S.ecol[e * nv + at[m]];
+      }
+    }
+    xv[m] = 0.0;
+    qv[m] = 0.0;
+    rv[m] = dv[m] = on ? b[q] : 0.0;
+    if (on) dir[q] = dv[m];
+    rr += rv[m] * rv[m];
   }
   rr = warp_sum(rr);
   __syncwarp();
@@ -196,60 +336,101 @@ __device__ inline int cg_warp(const CoarseSys& S, const double* b, double* x, do
   for (; it < max_it; ++it) {
     if (rr <= stop || rr == 0.0) break;
     double dq = 0.0;
-    for (int q = lane; q < nv; q += 32) {
-      const double aq = csr_row(S.aptr, S.acol, S.aval, q, d);
-      w[q] = aq;
-      dq += d[q] * aq;
+#pragma unroll
+    for (int m = 0; m < NR; ++m) {
+      double s = 0.0;
+      if (KEEP) {
+        double dn[CG_ROW];
+#pragma unroll
+        for (int e = 0; e < CG_ROW; ++e) dn[e] = dir[ac[e]];
+#pragma unroll
+        for (int e = 0; e < CG_ROW; ++e)
+          s += av[e] * dn[e];
+      }
+      for (int k = KEEP ? CG_ROW : 0; k < len[m]; k += CG_ROW) {
+        double a[CG_ROW], dn[CG_ROW];
+#pragma unroll
+        for (int e = 0; e < CG_ROW; ++e) {
+          a[e] = __ldg(S.eval + (k + e) * nv + at[m]);
+          dn[e] = dir[__ldg(S.ecol + (k + e) * nv + at[m])];
+        }
+#pragma unroll
+        for (int e = 0; e < CG_ROW; ++e)
+          if (k + e < len[m]) s += a[e] * dn[e];
+      }
+      if (lane + 32 * m >= nv) s = 0.0;
+      qv[m] = s;
+      dq += dv[m] * s;
     }
     dq = warp_sum(dq);
     if (dq == 0.0) break;
-    const double alpha = rr / dq;
+    double alpha, inv_rr;
+    div_and_rcp(rr, dq, rr, alpha, inv_rr);
     double rn = 0.0;
-    for (int q = lane; q < nv; q += 32) {
-      x[q] += alpha * d[q];
-      const double rq = r[q] - alpha * w[q];
-      r[q] = rq;
-      rn += rq * rq;
+#pragma unroll
+    for (int m = 0; m < NR; ++m) {
+      xv[m] += alpha * dv[m];
+      rv[m] -= alpha * qv[m];
+      rn += rv[m] * rv[m];
     }
     rn = warp_sum(rn);
-    const double beta = rn / rr;
-    // every lane has read d (the products above) before any lane rewrites it
-    __syncwarp();
-    for (int q = lane; q < nv; q += 32) d[q] = r[q] + beta * d[q];
+    const double beta = rn * inv_rr;
+    // every lane has read dir before any lane rewrites it (the sums above)
+#pragma unroll
+    for (int m = 0; m < NR; ++m) {
+      dv[m] = rv[m] + beta * dv[m];
+      if (lane + 32 * m < nv) dir[lane + 32 * m] = dv[m];
+    }
     __syncwarp();
     rr = rn;
   }
+#pragma unroll
+  for (int m = 0; m < NR; ++m)
+    if (lane + 32 * m < nv) x[lane + 32 * m] = xv[m];
   return it;
 }
 
-// Largest velocity block solved by one warp in the single-block solver.
-constexpr int WARP_CG_MAX_NV = 1024;
+// Largest velocity block solved by one warp in the single-block solver (four rows per lane).
+constexpr int WARP_CG_MAX_NV = 128;
 
 // z = P^{-1} v: CG on each velocity block, lumped mass on the pressure.  On a
 // single block with small blocks the three CG solves run concurrently, warp
 // w solving block w with warp-level synchronisation only; otherwise the team
-// runs them in lockstep (cg3).  cg holds 9 nv scratch entries.
+// runs them in lockstep (cg_team).  cg holds 9 nv scratch entries.
 __device__ inline int precond(const Ctx& C, const double* v, double* z, double* cg, int cg_max, double cg_rtol) {
   __shared__ int its_sh[3];
+  // search directions: of the three warp CGs, or of this CTA's rows in the team CG
+  __shared__ double dir_sh[CG_DIR];
   int its = 0;
   const int nv = C.S.nv;
   const int warp = threadIdx.x >> 5;
-  const bool par = !C.S.coupled && C.T.nblocks == 1 && blockDim.x >= 96 && nv <= WARP_CG_MAX_NV;
+  const bool par = !C.S.coupled && C.T.nblocks == 1 && blockDim.x >= 128 && nv <= WARP_CG_MAX_NV;
+  // the pressure part on the warps that no CG keeps busy
+  const int skip = par ? 96 : 0;
+  const int t0 = par ? (int)threadIdx.x - skip : (int)C.T.rank();
+  const int ts = (int)C.T.size() - skip;
+  if (t0 >= 0)
+    for (int q = t0; q < C.S.np; q += ts) z[3 * nv + q] = v[3 * nv + q] / C.S.mass[q];
   if (C.S.coupled) {
-    its = cg_coupled(C, v, z, cg, cg_max, cg_rtol);
+    its = cg_team<1>(C, v, z, cg, dir_sh, cg_max, cg_rtol);
   } else if (par) {
     if (warp < 3) {
-      const int n = cg_warp(C.S, v + warp * nv, z + warp * nv, cg + 3 * warp * nv, cg + (3 * warp + 1) * nv,
-                            cg + (3 * warp + 2) * nv, cg_max, cg_rtol);
+      const double* b = v + warp * nv;
+      double* x = z + warp * nv;
+      double* dir = dir_sh + warp * WARP_CG_MAX_NV;
+      const int n = nv <= 32   ? cg_warp<1>(C.S, b, x, dir, cg_max, cg_rtol)
+                    : nv <= 64 ? cg_warp<2>(C.S, b, x, dir, cg_max, cg_rtol)
+                               : cg_warp<4>(C.S, b, x, dir, cg_max, cg_rtol);
       if ((threadIdx.x & 31) == 0) its_sh[warp] = n;
     }
   } else {
-    its = cg3(C, v, z, cg, cg_max, cg_rtol);
+    its = cg_team<3>(C, v, z, cg, dir_sh, cg_max, cg_rtol);
   }
-  for (int q = (int)C.T.rank(); q < C.S.np; q += (int)C.T.size()) z[3 * nv + q] = v[3 * nv + q] / C.S.mass[q];
   C.T.sync();
-  if (par) its = its_sh[0] + its_sh[1] + its_sh[2];
-  C.T.sync();
+  if (par) {
+    its = its_sh[0] + its_sh[1] + its_sh[2];
+    C.T.sync();
+  }
   return its;
 }
 
@@ -257,7 +438,7 @@ __device__ inline int precond(const Ctx& C, const double* v, double* z, double* 
 // the coarsest level L (fields of type T, the solve in FP64); every thread of
 // the team must call it.  scratch: coarse_scratch_doubles(S) entries.
 template <class T>
-__device__ inline void minres_team(const Team& tm, const CoarseSys& S, const LevelDev<T>& L, double* scratch,
+__device__ __noinline__ void minres_team(const Team& tm, const CoarseSys& S, const LevelDev<T>& L, double* scratch,
                                    const CoarseParams& prm, double* info) {
   const int nv = S.nv, n = 3 * S.nv + S.np;
   Ctx C{S, tm, n};
@@ -308,33 +489,52 @@ __device__ inline void minres_team(const Team& tm, const CoarseSys& S, const Lev
 
   int iv_prev = 0, iv = 1, iv_next = 2, iz = 0, iz_next = 1, iw_prev = 0, iw = 1, iw_next = 2;
   int cg_total = precond(C, vv[iv], zz[iz], cg, prm.cg_max, prm.cg_rtol);
-  double gamma = sqrt(fmax(dot(C, zz[iz], vv[iv]), 0.0));
+  // the scalars of the recurrence are evaluated by the handler warp of each
+  // sum (team_reduce) and published; warps: those of a CTA with unknowns
+  const int warps = min((int)(blockDim.x >> 5), (n + 32 * (int)tm.nblocks - 1) / (32 * (int)tm.nblocks));
+  const double* g0 = team_reduce<1, 2>(C.T, dot_part(C, zz[iz], vv[iv]), warps, [](int, double tot, double* out) {
+    out[0] = sqrt(fmax(tot, 0.0));
+    out[1] = 1.0 / out[0];
+  });
+  double gamma = g0[0], inv_gamma = g0[1];
   int its = 0;
   double rel = 0.0;
   if (gamma > 0.0) {
     const double gamma1 = gamma;
-    double gamma_prev = 1.0, eta = gamma;
+    double inv_gamma_prev = 1.0, eta = gamma;
     double c_prev = 1.0, cc = 1.0, s_prev = 0.0, ss = 0.0;
     for (; its < prm.minres_max;) {
-      for (int q = (int)tm.rank(); q < n; q += (int)tm.size()) zz[iz][q] /= gamma;
+      for (int q = (int)tm.rank(); q < n; q += (int)tm.size()) zz[iz][q] *= inv_gamma;
       tm.sync();
       applyK(C, zz[iz], Kz);
-      const double delta = dot(C, Kz, zz[iz]);
-      const double r1 = delta / gamma, r2 = gamma / gamma_prev;
+      const double* r = team_reduce<1, 2>(C.T, dot_part(C, Kz, zz[iz]), warps, [=](int, double tot, double* out) {
+        out[0] = tot;
+        out[1] = tot * inv_gamma;
+      });
+      const double delta = r[0], r1 = r[1], r2 = gamma * inv_gamma_prev;
       for (int q = (int)tm.rank(); q < n; q += (int)tm.size())
         vv[iv_next][q] = Kz[q] - r1 * vv[iv][q] - r2 * vv[iv_prev][q];
       tm.sync();
       cg_total += precond(C, vv[iv_next], zz[iz_next], cg, prm.cg_max, prm.cg_rtol);
-      const double gamma_next = sqrt(fmax(dot(C, zz[iz_next], vv[iv_next]), 0.0));
-      const double a0 = cc * delta - c_prev * ss * gamma;
-      const double a1 = sqrt(a0 * a0 + gamma_next * gamma_next);
-      const double a2 = ss * delta + c_prev * cc * gamma;
-      const double a3 = s_prev * gamma;
+      const double* g =
+          team_reduce<1, 6>(C.T, dot_part(C, zz[iz_next], vv[iv_next]), warps, [=](int, double tot, double* out) {
+            const double gamma_next = sqrt(fmax(tot, 0.0));
+            const double a0 = cc * delta - c_prev * ss * gamma;
+            const double a1 = sqrt(a0 * a0 + gamma_next * gamma_next);
+            const double inv_a1 = 1.0 / a1;
+            out[0] = gamma_next;
+            out[1] = 1.0 / gamma_next;
+            out[2] = a1;
+            out[3] = inv_a1;
+            out[4] = a0 * inv_a1;
+            out[5] = gamma_next * inv_a1;
+          });
+      const double gamma_next = g[0], inv_gamma_next = g[1], a1 = g[2], inv_a1 = g[3], c_next = g[4], s_next = g[5];
       if (a1 == 0.0) break;
-      const double c_next = a0 / a1, s_next = gamma_next / a1;
+      const double a2 = ss * delta + c_prev * cc * gamma, a3 = s_prev * gamma;
       const double step = c_next * eta;
       for (int q = (int)tm.rank(); q < n; q += (int)tm.size()) {
-        const double wn = (zz[iz][q] - a3 * ww[iw_prev][q] - a2 * ww[iw][q]) / a1;
+        const double wn = (zz[iz][q] - a3 * ww[iw_prev][q] - a2 * ww[iw][q]) * inv_a1;
         ww[iw_next][q] = wn;
         x[q] += step * wn;
       }
@@ -353,15 +553,17 @@ __device__ inline void minres_team(const Team& tm, const CoarseSys& S, const Lev
       iw_prev = iw;
       iw = iw_next;
       iw_next = t;
-      gamma_prev = gamma;
+      inv_gamma_prev = inv_gamma;
       gamma = gamma_next;
+      inv_gamma = inv_gamma_next;
       c_prev = cc;
       cc = c_next;
       s_prev = ss;
       ss = s_next;
-      rel = fabs(eta) / gamma1;
+      rel = eta;
       if (fabs(eta) <= prm.minres_rtol * gamma1 || gamma == 0.0) break;
     }
+    rel = fabs(rel) / gamma1;
   }
   // (U, P) += x
   for (int q = (int)tm.rank(); q < n; q += (int)tm.size()) {

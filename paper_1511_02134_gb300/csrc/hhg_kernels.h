@@ -201,6 +201,9 @@ struct CoarseSys {
   const int32_t* aptr;    // scalar A in CSR, nv rows
   const int32_t* acol;
   const double* aval;
+  const int32_t* ecol;    // A again with its rows side by side, entry e of row r at e rows + r (a thread
+  const double* eval;     // per row then reads coalesced), padded with zeros on the diagonal to a multiple
+                          // of COARSE_ELL_ROUND entries; null above COARSE_ELL_MAX_ROWS rows
   const double* mass;     // lumped mass of each pressure unknown
 };
 struct CoarseParams {
@@ -213,10 +216,12 @@ struct CoarseParams {
 __host__ __device__ inline int64_t coarse_scratch_doubles(const CoarseSys& S) {
   return 11 * (3 * (int64_t)S.nv + S.np) + 9 * (int64_t)S.nv;
 }
+constexpr int32_t COARSE_ELL_ROUND = 8;
+constexpr int32_t COARSE_ELL_MAX_ROWS = 8192;  // 16 CTAs of 512 threads, one row each
 // A coarsest level this small is solved by one thread block (one warp per CG).
-constexpr int64_t COARSE_BLOCK_MAX_UNKNOWNS = 4096;
+constexpr int32_t COARSE_BLOCK_MAX_NV = 128;
 __host__ __device__ inline bool coarse_fits_block(const CoarseSys& S) {
-  return 3 * (int64_t)S.nv + S.np <= COARSE_BLOCK_MAX_UNKNOWNS;
+  return S.nv <= COARSE_BLOCK_MAX_NV;
 }
 template <class T>
 void launch_coarse_solve(const CoarseSys& S, const LevelDev<T>& L, double* scratch, CoarseParams prm, double* info,
