@@ -289,6 +289,7 @@ template <int NSYS>
 __device__ inline int cg_team(const Ctx& C, const double* b, double* x, double* cg, double* dir, int max_it,
                               double rtol) {
   const int N = NSYS == 3 ? C.S.nv : 3 * C.S.nv;
+  if (N == 0) return 0;  // no velocity unknown (the unit cube's level 0): A has no rows
   const int rc = (N + (int)C.T.nblocks - 1) / (int)C.T.nblocks;
   if (C.S.eval && NSYS * ((rc + 31) / 32 * 32) <= min((int)blockDim.x, CG_DIR))
     return cg_team_regs<NSYS>(C, b, x, dir, max_it, rtol);
@@ -404,7 +405,7 @@ __device__ inline int precond(const Ctx& C, const double* v, double* z, double* 
   int its = 0;
   const int nv = C.S.nv;
   const int warp = threadIdx.x >> 5;
-  const bool par = !C.S.coupled && C.T.nblocks == 1 && blockDim.x >= 128 && nv <= WARP_CG_MAX_NV;
+  const bool par = !C.S.coupled && C.T.nblocks == 1 && blockDim.x >= 128 && nv <= WARP_CG_MAX_NV && nv > 0;
   // the pressure part on the warps that no CG keeps busy
   const int skip = par ? 96 : 0;
   const int t0 = par ? (int)threadIdx.x - skip : (int)C.T.rank();

@@ -25,6 +25,8 @@ def pkg():
 
 # (cells, level, form, slip sides): free velocity nodes, prod(cells 2^level - 1) without slip
 SHAPES = [
+    ((1, 1, 1), 0, 0, ()),          # none: pressure unknowns only
+    ((2, 1, 1), 0, 1, ()),
     ((1, 1, 1), 1, 0, ()),          # 1
     ((1, 1, 1), 2, 0, ()),          # 27: one row per lane
     ((2, 1, 1), 2, 0, ()),          # 63: two
@@ -63,6 +65,6 @@ def test_coarse_solve_shapes(pkg, cells, level, form, slip, zero):
     MG.vcycle(H, level, u, p, f, g)  # on the coarsest level: the MINRES correction
     gu = u_from_lattice(L, dims, mesh.level_field(level, "U"))
     gp = p_from_lattice(L, dims, mesh.level_field(level, "P"))
-    assert rel_err(gu, u) < 1e-9
+    assert L.n_u == 0 or rel_err(gu, u) < 1e-9
     assert rel_err(L.project_pressure(gp), L.project_pressure(p)) < 1e-9
     mesh.close()
