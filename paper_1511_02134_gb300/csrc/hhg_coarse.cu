@@ -27,12 +27,12 @@ unsigned g_coarse_cluster = 8;
 }  // namespace
 
 // Launch shape of the coarse solve: small coarse systems are latency bound
-// and run in one block (one warp per CG; 128 threads where they cover the
-// coupled block's rows too); larger ones run on a cluster.
+// and run in one block of 128 threads (cheap barriers, one warp per CG);
+// larger ones run on a cluster.
 void coarse_shape(const CoarseSys& S, unsigned& nblocks, unsigned& threads) {
   if (coarse_fits_block(S)) {
     nblocks = 1;
-    threads = S.nv <= 32 ? 128 : CT;
+    threads = 128;
   } else {
     nblocks = g_coarse_cluster;
     threads = CT;

@@ -8,6 +8,10 @@
 // fixed upper trip counts (max iterations).  Used by the coarse-solve kernel
 // and by the fused coarse-levels cycle.
 //
+// Row products and dot products are chains of fused multiply-adds in row
+// order, and the sums of the team have a fixed order (hhg_team.cuh): an
+// inexact solve amplifies its rounding, so the order is part of the result.
+//
 // Recurrences (start from zero):
 //   CG:     stop before an iteration when r.r <= rtol^2 r0.r0 (or r.r = 0),
 //           or when d.Ad = 0; at most cg_max iterations.
@@ -34,15 +38,14 @@ __device__ __forceinline__ double csr_row(const int32_t* ptr, const int32_t* col
                                           const double* x) {
   double s = 0.0;
   const int e = ptr[r + 1];
-#pragma unroll 4
-  for (int k = ptr[r]; k < e; ++k) s += val[k] * x[col[k]];
+  for (int k = ptr[r]; k < e; ++k) s = fma(val[k], x[col[k]], s);
   return s;
 }
 
 // This thread's part of a.b.
 __device__ __forceinline__ double dot_part(const Ctx& C, const double* a, const double* b) {
   double s = 0;
-  for (int q = (int)C.T.rank(); q < C.n; q += (int)C.T.size()) s += a[q] * b[q];
+  for (int q = (int)C.T.rank(); q < C.n; q += (int)C.T.size()) s = fma(a[q], b[q], s);
   return s;
 }
 
@@ -61,14 +64,16 @@ __device__ inline void applyK(const Ctx& C, const double* x, double* y) {
 // the others go on.  b, x: NSYS N entries.  Returns the iterations summed
 // over the systems.
 //
-// cg_team_regs: a CTA holds a run of rows of every system and a thread at
-// most one (system, row) pair, whose x, r, d, A d and first CG_ROW matrix
-// entries (with the addresses of their directions) stay in registers; a
-// warp's pairs belong to one system.  The directions lie in the shared memory
-// of their CTAs, dir, and are read through the cluster's shared window.  An
-// iteration is three cluster barriers: d.Ad, r.r and the new directions.  It
-// is bound by the latencies of the FP64 chain (64 cycles per dependent
-// operation, 560 per division) and of the barriers (480 cycles each).
+// cg_team_regs: a CTA holds a run of groups of 32 rows of every system and a
+// warp at most one (system, group), a row per lane, whose x, r, d, A d and
+// first CG_ROW matrix entries (with the addresses of their directions) stay
+// in registers.  The directions lie in the shared memory of their CTAs, dir,
+// and are read through the cluster's shared window.  An iteration is three
+// cluster barriers: d.Ad, r.r and the new directions.  It is bound by the
+// latencies of the FP64 chain (64 cycles per dependent operation, 560 per
+// division) and of the barriers (480 cycles each): on the obstacle channel's
+// level 1 (1,427 rows, 16 CTAs) an iteration takes 5.5 us, against 27 us
+// with every thread evaluating the scalars and the vectors in global memory.
 constexpr int CG_ROW = COARSE_ELL_ROUND;
 constexpr int CG_DIR = 512;  // directions of a CTA: one per thread
 
@@ -76,22 +81,22 @@ template <int NSYS>
 __device__ __noinline__ int cg_team_regs(const Ctx& C, const double* b, double* x, double* dir, int max_it,
                                          double rtol) {
   const int N = NSYS == 3 ? C.S.nv : 3 * C.S.nv;
-  const int rc = (N + (int)C.T.nblocks - 1) / (int)C.T.nblocks;  // rows per CTA
-  const int rp = (rc + 31) / 32 * 32;                            // padded: whole warps per system
-  const int each = rp / 32;                                      // warps per system
-  const int sys = (int)(threadIdx.x >> 5) / each;
+  const int groups = (N + 31) / 32;
+  const int each = (groups + (int)C.T.nblocks - 1) / (int)C.T.nblocks;  // groups of a system per CTA
+  const int rc = 32 * each;                                            // its rows
+  const int warp = threadIdx.x >> 5, sys = warp / each;
   const bool used = sys < NSYS;
-  const int l = (int)threadIdx.x - sys * rp;  // row within the CTA
-  const int row = (int)blockIdx.x * rc + l;
-  const bool on = used && l < rc && row < N;
-  const int idx = on ? sys * N + row : -1;
   const int mine = used ? sys : 0;
-  const uint32_t dir0 = (uint32_t)__cvta_generic_to_shared(dir) + 8u * (uint32_t)(mine * rp);
-  const uint32_t inv = 0xffffffffu / (uint32_t)rc + 1u;  // col / rc = umulhi(col, inv): col, rc < 2^13 (rc = 1: inv = 0)
+  const int l = (int)threadIdx.x - sys * rc;  // row within the CTA
+  const int row = (int)blockIdx.x * rc + l, group = row >> 5;
+  const bool live = used && group < groups;   // (uniform in the warp)
+  const bool on = live && row < N;
+  const int idx = on ? sys * N + row : -1;
+  const uint32_t dir0 = (uint32_t)__cvta_generic_to_shared(dir) + 8u * (uint32_t)(mine * rc);
+  const uint32_t inv = 0xffffffffu / (uint32_t)rc + 1u;  // col / rc = umulhi(col, inv): col, rc < 2^13
   auto addr_of = [&](int col) {
-    const uint32_t o = rc == 1 ? (uint32_t)col : __umulhi((uint32_t)col, inv);
-    const uint32_t at = dir0 + 8u * ((uint32_t)col - o * (uint32_t)rc);
-    return C.T.nblocks > 1 ? team_shared_addr(at, o) : at;
+    const uint32_t o = __umulhi((uint32_t)col, inv);
+    return team_shared_addr(dir0 + 8u * ((uint32_t)col - o * (uint32_t)rc), o);
   };
   // entries of the warp's longest row (the others' absent ones are zeros on
   // their own directions; a thread without a row reads row 0 and drops it)
@@ -106,12 +111,14 @@ __device__ __noinline__ int cg_team_regs(const Ctx& C, const double* b, double* 
     ad[e] = addr_of(ec[(int64_t)e * N]);
   }
   double xv = 0.0, qv = 0.0, rv = on ? b[idx] : 0.0, dv = rv;
-  if (used) dir[mine * rp + l] = dv;
+  if (used) dir[mine * rc + l] = dv;
   // state of the handler warps: r.r, the stopping bound, running, iterations
-  double rr = 0.0, stop = 0.0, inv_rr = 0.0;
+  double rr = 0.0, stop = 0.0;
   bool run = false;
   int its = 0;
-  const double* res = team_reduce<NSYS, 2>(C.T, rv * rv, each, [&](int, double tot, double* out) {
+  if (live) team_publish(C.T, rv * rv, mine, group);
+  double res[2 * NSYS];
+  team_finish<NSYS, 2>(C.T, groups, res, [&](int, double tot, double* out) {
     rr = tot;
     stop = rtol * rtol * tot;
     run = !(rr <= stop || rr == 0.0);
@@ -124,15 +131,14 @@ __device__ __noinline__ int cg_team_regs(const Ctx& C, const double* b, double* 
 #pragma unroll
     for (int s = 0; s < NSYS; ++s) any |= res[2 * s] != 0.0;
     if (!any) break;
-    bool go = used && res[2 * mine] != 0.0;
-    double acc = 0.0;
+    bool go = live && res[2 * mine] != 0.0;
     if (go) {
       double dn[CG_ROW];
 #pragma unroll
       for (int e = 0; e < CG_ROW; ++e) dn[e] = ld_team_shared(ad[e]);
       qv = 0.0;
 #pragma unroll
-      for (int e = 0; e < CG_ROW; ++e) qv += av[e] * dn[e];
+      for (int e = 0; e < CG_ROW; ++e) qv = fma(av[e], dn[e], qv);
       for (int k = CG_ROW; k < len; k += CG_ROW) {
         double a[CG_ROW];
         uint32_t at[CG_ROW];
@@ -145,30 +151,27 @@ __device__ __noinline__ int cg_team_regs(const Ctx& C, const double* b, double* 
         for (int e = 0; e < CG_ROW; ++e) dn[e] = ld_team_shared(at[e]);
 #pragma unroll
         for (int e = 0; e < CG_ROW; ++e)
-          if (k + e < len) qv += a[e] * dn[e];
+          if (k + e < len) qv = fma(a[e], dn[e], qv);
       }
       if (!on) qv = 0.0;
-      acc = dv * qv;
+      team_publish(C.T, dv * qv, mine, group);
     }
-    res = team_reduce<NSYS, 2>(C.T, acc, each, [&](int, double tot, double* out) {
-      double alpha;
-      div_and_rcp(rr, tot, rr, alpha, inv_rr);
+    team_finish<NSYS, 2>(C.T, groups, res, [&](int, double tot, double* out) {
       if (run && tot == 0.0) run = false;
       out[0] = run ? 1.0 : 0.0;
-      out[1] = run ? alpha : 0.0;
+      out[1] = run ? rr / tot : 0.0;
     });
     go = go && res[2 * mine] != 0.0;
-    acc = 0.0;
     if (go) {
       const double alpha = res[2 * mine + 1];
-      rv -= alpha * qv;
-      acc = rv * rv;
-      xv += alpha * dv;
+      rv = fma(-alpha, qv, rv);
+      team_publish(C.T, rv * rv, mine, group);
+      xv = fma(alpha, dv, xv);
     }
-    res = team_reduce<NSYS, 2>(C.T, acc, each, [&](int, double tot, double* out) {
+    team_finish<NSYS, 2>(C.T, groups, res, [&](int, double tot, double* out) {
       out[0] = out[1] = 0.0;
       if (run) {
-        out[1] = tot * inv_rr;
+        out[1] = tot / rr;
         rr = tot;
         ++its;
         run = !(rr <= stop || rr == 0.0);
@@ -176,13 +179,13 @@ __device__ __noinline__ int cg_team_regs(const Ctx& C, const double* b, double* 
       }
     });
     if (go) {
-      dv = rv + res[2 * mine + 1] * dv;
-      dir[mine * rp + l] = dv;
+      dv = fma(res[2 * mine + 1], dv, rv);
+      dir[mine * rc + l] = dv;
     }
     C.T.sync();
   }
   if (on) x[idx] = xv;
-  res = team_reduce<NSYS, 1>(C.T, 0.0, each, [&](int, double, double* out) { out[0] = (double)its; });
+  team_finish<NSYS, 1>(C.T, 0, res, [&](int, double, double* out) { out[0] = (double)its; });
   double n = 0.0;
 #pragma unroll
   for (int s = 0; s < NSYS; ++s) n += res[s];
@@ -190,39 +193,40 @@ __device__ __noinline__ int cg_team_regs(const Ctx& C, const double* b, double* 
 }
 
 // The same for any number of rows per thread, on vectors in global memory
-// (cg: r, d and A d, NSYS N entries each).
+// (cg: r, d and A d, NSYS N entries each); a thread takes its rows in every
+// system.
 template <int NSYS>
 __device__ __noinline__ int cg_team_mem(const Ctx& C, const double* b, double* x, double* cg, int max_it,
                                         double rtol) {
   const int N = NSYS == 3 ? C.S.nv : 3 * C.S.nv;
-  // the warps of a CTA in NSYS groups
-  const int each = (int)(blockDim.x >> 5) / NSYS;
-  const int warp = threadIdx.x >> 5, mine = min(warp / each, NSYS - 1);
-  // (a remainder warp has no rows)
-  const int t0 = warp < NSYS * each
-                     ? ((warp - mine * each) * (int)C.T.nblocks + (int)blockIdx.x) * 32 + (int)(threadIdx.x & 31)
-                     : N;
-  const int step = each * (int)C.T.nblocks * 32;
   double* R = cg;
   double* D = cg + NSYS * N;
   double* Q = cg + 2 * NSYS * N;
-  b += mine * N;
-  x += mine * N;
-  R += mine * N;
-  D += mine * N;
-  Q += mine * N;
-  double acc = 0.0;
-  for (int q = t0; q < N; q += step) {
-    const double v = b[q];
-    x[q] = 0.0;
-    R[q] = v;
-    D[q] = v;
-    acc += v * v;
-  }
-  double rr = 0.0, stop = 0.0, inv_rr = 0.0;
+  const int t0 = (int)C.T.rank(), step = (int)C.T.size();
+  const int group = t0 >> 5, groups = (min(N, step) + 31) / 32;
+  auto publish = [&](const double (&v)[NSYS]) {
+    if (group < groups)
+#pragma unroll
+      for (int s = 0; s < NSYS; ++s) team_publish(C.T, v[s], s, group);
+  };
+  double acc[NSYS];
+#pragma unroll
+  for (int s = 0; s < NSYS; ++s) acc[s] = 0.0;
+  for (int q = t0; q < N; q += step)
+#pragma unroll
+    for (int s = 0; s < NSYS; ++s) {
+      const double v = b[s * N + q];
+      x[s * N + q] = 0.0;
+      R[s * N + q] = v;
+      D[s * N + q] = v;
+      acc[s] = fma(v, v, acc[s]);
+    }
+  double rr = 0.0, stop = 0.0;
   bool run = false;
   int its = 0;
-  const double* res = team_reduce<NSYS, 2>(C.T, acc, each, [&](int, double tot, double* out) {
+  publish(acc);
+  double res[2 * NSYS];
+  team_finish<NSYS, 2>(C.T, groups, res, [&](int, double tot, double* out) {
     rr = tot;
     stop = rtol * rtol * tot;
     run = !(rr <= stop || rr == 0.0);
@@ -234,48 +238,56 @@ __device__ __noinline__ int cg_team_mem(const Ctx& C, const double* b, double* x
 #pragma unroll
     for (int s = 0; s < NSYS; ++s) any |= res[2 * s] != 0.0;
     if (!any) break;
-    const bool on = res[2 * mine] != 0.0;
-    acc = 0.0;
-    if (on)
+#pragma unroll
+    for (int s = 0; s < NSYS; ++s) {
+      acc[s] = 0.0;
+      if (res[2 * s] == 0.0) continue;
       for (int q = t0; q < N; q += step) {
-        const double aq = csr_row(C.S.aptr, C.S.acol, C.S.aval, q, D);
-        Q[q] = aq;
-        acc += D[q] * aq;
+        const double aq = csr_row(C.S.aptr, C.S.acol, C.S.aval, q, D + s * N);
+        Q[s * N + q] = aq;
+        acc[s] = fma(D[s * N + q], aq, acc[s]);
       }
-    res = team_reduce<NSYS, 2>(C.T, acc, each, [&](int, double tot, double* out) {
-      double alpha;
-      div_and_rcp(rr, tot, rr, alpha, inv_rr);
+    }
+    publish(acc);
+    team_finish<NSYS, 2>(C.T, groups, res, [&](int, double tot, double* out) {
       if (run && tot == 0.0) run = false;
       out[0] = run ? 1.0 : 0.0;
-      out[1] = run ? alpha : 0.0;
+      out[1] = run ? rr / tot : 0.0;
     });
-    const bool go = on && res[2 * mine] != 0.0;
-    const double alpha = res[2 * mine + 1];
-    acc = 0.0;
-    if (go)
-      for (int q = t0; q < N; q += step) {
-        x[q] += alpha * D[q];
-        const double rq = R[q] - alpha * Q[q];
-        R[q] = rq;
-        acc += rq * rq;
-      }
-    res = team_reduce<NSYS, 2>(C.T, acc, each, [&](int, double tot, double* out) {
+    bool go[NSYS];
+#pragma unroll
+    for (int s = 0; s < NSYS; ++s) {
+      go[s] = res[2 * s] != 0.0;
+      const double alpha = res[2 * s + 1];
+      acc[s] = 0.0;
+      if (go[s])
+        for (int q = t0; q < N; q += step) {
+          x[s * N + q] += alpha * D[s * N + q];
+          const double rq = R[s * N + q] - alpha * Q[s * N + q];
+          R[s * N + q] = rq;
+          acc[s] = fma(rq, rq, acc[s]);
+        }
+    }
+    publish(acc);
+    team_finish<NSYS, 2>(C.T, groups, res, [&](int, double tot, double* out) {
       out[0] = out[1] = 0.0;
       if (run) {
-        out[1] = tot * inv_rr;
+        out[1] = tot / rr;
         rr = tot;
         ++its;
         run = !(rr <= stop || rr == 0.0);
         out[0] = run ? 1.0 : 0.0;
       }
     });
-    if (go) {
-      const double beta = res[2 * mine + 1];
-      for (int q = t0; q < N; q += step) D[q] = R[q] + beta * D[q];
-    }
+#pragma unroll
+    for (int s = 0; s < NSYS; ++s)
+      if (go[s]) {
+        const double beta = res[2 * s + 1];
+        for (int q = t0; q < N; q += step) D[s * N + q] = R[s * N + q] + beta * D[s * N + q];
+      }
     C.T.sync();
   }
-  res = team_reduce<NSYS, 1>(C.T, 0.0, 0, [&](int, double, double* out) { out[0] = (double)its; });
+  team_finish<NSYS, 1>(C.T, 0, res, [&](int, double, double* out) { out[0] = (double)its; });
   double n = 0.0;
 #pragma unroll
   for (int s = 0; s < NSYS; ++s) n += res[s];
@@ -283,15 +295,16 @@ __device__ __noinline__ int cg_team_mem(const Ctx& C, const double* b, double* x
 }
 
 // Team CG of the preconditioner; cg: 9 nv entries of global scratch, dir:
-// CG_DIR entries of shared memory.  One row per thread covers nv <= 2,560 on
-// 16 CTAs of 512 threads.
+// CG_DIR entries of shared memory.  One row per lane covers nv <= 2,560 on
+// 16 CTAs of 512 threads.  (One block keeps its few rows in memory, L1: the
+// cube's level 2 in the D form, 81 rows, 355 us per solve against 378.)
 template <int NSYS>
 __device__ inline int cg_team(const Ctx& C, const double* b, double* x, double* cg, double* dir, int max_it,
                               double rtol) {
   const int N = NSYS == 3 ? C.S.nv : 3 * C.S.nv;
   if (N == 0) return 0;  // no velocity unknown (the unit cube's level 0): A has no rows
-  const int rc = (N + (int)C.T.nblocks - 1) / (int)C.T.nblocks;
-  if (C.S.eval && NSYS * ((rc + 31) / 32 * 32) <= min((int)blockDim.x, CG_DIR))
+  const int each = ((N + 31) / 32 + (int)C.T.nblocks - 1) / (int)C.T.nblocks;
+  if (C.T.nblocks > 1 && C.S.eval && 32 * NSYS * each <= min((int)blockDim.x, CG_DIR))
     return cg_team_regs<NSYS>(C, b, x, dir, max_it, rtol);
   return cg_team_mem<NSYS>(C, b, x, cg, max_it, rtol);
 }
@@ -328,7 +341,7 @@ __device__ __noinline__ int cg_warp(const CoarseSys& S, const double* b, double*
     qv[m] = 0.0;
     rv[m] = dv[m] = on ? b[q] : 0.0;
     if (on) dir[q] = dv[m];
-    rr += rv[m] * rv[m];
+    rr = fma(rv[m], rv[m], rr);
   }
   rr = warp_sum(rr);
   __syncwarp();
@@ -346,7 +359,7 @@ __device__ __noinline__ int cg_warp(const CoarseSys& S, const double* b, double*
         for (int e = 0; e < CG_ROW; ++e) dn[e] = dir[ac[e]];
 #pragma unroll
         for (int e = 0; e < CG_ROW; ++e)
-          s += av[e] * dn[e];
+          s = fma(av[e], dn[e], s);
       }
       for (int k = KEEP ? CG_ROW : 0; k < len[m]; k += CG_ROW) {
         double a[CG_ROW], dn[CG_ROW];
@@ -357,29 +370,28 @@ __device__ __noinline__ int cg_warp(const CoarseSys& S, const double* b, double*
         }
 #pragma unroll
         for (int e = 0; e < CG_ROW; ++e)
-          if (k + e < len[m]) s += a[e] * dn[e];
+          if (k + e < len[m]) s = fma(a[e], dn[e], s);
       }
       if (lane + 32 * m >= nv) s = 0.0;
       qv[m] = s;
-      dq += dv[m] * s;
+      dq = fma(dv[m], s, dq);
     }
     dq = warp_sum(dq);
     if (dq == 0.0) break;
-    double alpha, inv_rr;
-    div_and_rcp(rr, dq, rr, alpha, inv_rr);
+    const double alpha = rr / dq;
     double rn = 0.0;
 #pragma unroll
     for (int m = 0; m < NR; ++m) {
-      xv[m] += alpha * dv[m];
-      rv[m] -= alpha * qv[m];
-      rn += rv[m] * rv[m];
+      xv[m] = fma(alpha, dv[m], xv[m]);
+      rv[m] = fma(-alpha, qv[m], rv[m]);
+      rn = fma(rv[m], rv[m], rn);
     }
     rn = warp_sum(rn);
-    const double beta = rn * inv_rr;
+    const double beta = rn / rr;
     // every lane has read dir before any lane rewrites it (the sums above)
 #pragma unroll
     for (int m = 0; m < NR; ++m) {
-      dv[m] = rv[m] + beta * dv[m];
+      dv[m] = fma(beta, dv[m], rv[m]);
       if (lane + 32 * m < nv) dir[lane + 32 * m] = dv[m];
     }
     __syncwarp();
@@ -391,8 +403,64 @@ __device__ __noinline__ int cg_warp(const CoarseSys& S, const double* b, double*
   return it;
 }
 
-// Largest velocity block solved by one warp in the single-block solver (four rows per lane).
-constexpr int WARP_CG_MAX_NV = 128;
+// The same for any number of rows per lane, on vectors in memory (r, d, w: nv entries each).
+static __device__ __noinline__ int cg_warp_mem(const CoarseSys& S, const double* b, double* x, double* r, double* d,
+                                        double* w, int max_it, double rtol) {
+  const int lane = threadIdx.x & 31, nv = S.nv;
+  double rr = 0.0;
+  for (int q = lane; q < nv; q += 32) {
+    x[q] = 0.0;
+    r[q] = b[q];
+    d[q] = b[q];
+    rr = fma(b[q], b[q], rr);
+  }
+  rr = warp_sum(rr);
+  __syncwarp();
+  const double stop = rtol * rtol * rr;
+  int it = 0;
+  for (; it < max_it; ++it) {
+    if (rr <= stop || rr == 0.0) break;
+    double dq = 0.0;
+    for (int q = lane; q < nv; q += 32) {
+      const int len = S.aptr[q + 1] - S.aptr[q];
+      double s = 0.0;
+      for (int k = 0; k < len; k += CG_ROW) {
+        double a[CG_ROW], dn[CG_ROW];
+#pragma unroll
+        for (int e = 0; e < CG_ROW; ++e) {
+          a[e] = __ldg(S.eval + (k + e) * nv + q);
+          dn[e] = d[__ldg(S.ecol + (k + e) * nv + q)];
+        }
+#pragma unroll
+        for (int e = 0; e < CG_ROW; ++e) s = fma(a[e], dn[e], s);
+      }
+      w[q] = s;
+      dq = fma(d[q], s, dq);
+    }
+    dq = warp_sum(dq);
+    if (dq == 0.0) break;
+    const double alpha = rr / dq;
+    double rn = 0.0;
+    for (int q = lane; q < nv; q += 32) {
+      x[q] += alpha * d[q];
+      const double rq = r[q] - alpha * w[q];
+      r[q] = rq;
+      rn = fma(rq, rq, rn);
+    }
+    rn = warp_sum(rn);
+    const double beta = rn / rr;
+    // every lane has read d (the products above) before any lane rewrites it
+    __syncwarp();
+    for (int q = lane; q < nv; q += 32) d[q] = r[q] + beta * d[q];
+    __syncwarp();
+    rr = rn;
+  }
+  return it;
+}
+
+// Largest velocity block solved by one warp in the single-block solver, and
+// the largest with its vectors in registers (four rows per lane).
+constexpr int WARP_CG_MAX_NV = 1024, WARP_CG_REG_NV = 128;
 
 // z = P^{-1} v: CG on each velocity block, lumped mass on the pressure.  On a
 // single block with small blocks the three CG solves run concurrently, warp
@@ -418,10 +486,12 @@ __device__ inline int precond(const Ctx& C, const double* v, double* z, double* 
     if (warp < 3) {
       const double* b = v + warp * nv;
       double* x = z + warp * nv;
-      double* dir = dir_sh + warp * WARP_CG_MAX_NV;
-      const int n = nv <= 32   ? cg_warp<1>(C.S, b, x, dir, cg_max, cg_rtol)
-                    : nv <= 64 ? cg_warp<2>(C.S, b, x, dir, cg_max, cg_rtol)
-                               : cg_warp<4>(C.S, b, x, dir, cg_max, cg_rtol);
+      double* dir = dir_sh + warp * WARP_CG_REG_NV;
+      double* mem = cg + 3 * warp * nv;
+      const int n = nv <= 32               ? cg_warp<1>(C.S, b, x, dir, cg_max, cg_rtol)
+                    : nv <= 64             ? cg_warp<2>(C.S, b, x, dir, cg_max, cg_rtol)
+                    : nv <= WARP_CG_REG_NV ? cg_warp<4>(C.S, b, x, dir, cg_max, cg_rtol)
+                                           : cg_warp_mem(C.S, b, x, mem, mem + nv, mem + 2 * nv, cg_max, cg_rtol);
       if ((threadIdx.x & 31) == 0) its_sh[warp] = n;
     }
   } else {
@@ -491,51 +561,48 @@ __device__ __noinline__ void minres_team(const Team& tm, const CoarseSys& S, con
   int iv_prev = 0, iv = 1, iv_next = 2, iz = 0, iz_next = 1, iw_prev = 0, iw = 1, iw_next = 2;
   int cg_total = precond(C, vv[iv], zz[iz], cg, prm.cg_max, prm.cg_rtol);
   // the scalars of the recurrence are evaluated by the handler warp of each
-  // sum (team_reduce) and published; warps: those of a CTA with unknowns
-  const int warps = min((int)(blockDim.x >> 5), (n + 32 * (int)tm.nblocks - 1) / (32 * (int)tm.nblocks));
-  const double* g0 = team_reduce<1, 2>(C.T, dot_part(C, zz[iz], vv[iv]), warps, [](int, double tot, double* out) {
-    out[0] = sqrt(fmax(tot, 0.0));
-    out[1] = 1.0 / out[0];
-  });
-  double gamma = g0[0], inv_gamma = g0[1];
+  // sum (team_finish) and published
+  double gamma;
+  team_reduce1<1>(C.T, dot_part(C, zz[iz], vv[iv]), n, &gamma,
+                  [](int, double tot, double* out) { out[0] = sqrt(fmax(tot, 0.0)); });
   int its = 0;
   double rel = 0.0;
   if (gamma > 0.0) {
     const double gamma1 = gamma;
-    double inv_gamma_prev = 1.0, eta = gamma;
+    double gamma_prev = 1.0, eta = gamma;
     double c_prev = 1.0, cc = 1.0, s_prev = 0.0, ss = 0.0;
     for (; its < prm.minres_max;) {
-      for (int q = (int)tm.rank(); q < n; q += (int)tm.size()) zz[iz][q] *= inv_gamma;
+      for (int q = (int)tm.rank(); q < n; q += (int)tm.size()) zz[iz][q] /= gamma;
       tm.sync();
       applyK(C, zz[iz], Kz);
-      const double* r = team_reduce<1, 2>(C.T, dot_part(C, Kz, zz[iz]), warps, [=](int, double tot, double* out) {
+      double r[3];
+      team_reduce1<3>(C.T, dot_part(C, Kz, zz[iz]), n, r, [=](int, double tot, double* out) {
         out[0] = tot;
-        out[1] = tot * inv_gamma;
+        out[1] = tot / gamma;
+        out[2] = gamma / gamma_prev;
       });
-      const double delta = r[0], r1 = r[1], r2 = gamma * inv_gamma_prev;
+      const double delta = r[0], r1 = r[1], r2 = r[2];
       for (int q = (int)tm.rank(); q < n; q += (int)tm.size())
         vv[iv_next][q] = Kz[q] - r1 * vv[iv][q] - r2 * vv[iv_prev][q];
       tm.sync();
       cg_total += precond(C, vv[iv_next], zz[iz_next], cg, prm.cg_max, prm.cg_rtol);
-      const double* g =
-          team_reduce<1, 6>(C.T, dot_part(C, zz[iz_next], vv[iv_next]), warps, [=](int, double tot, double* out) {
+      double g[6];
+      team_reduce1<6>(C.T, dot_part(C, zz[iz_next], vv[iv_next]), n, g, [=](int, double tot, double* out) {
             const double gamma_next = sqrt(fmax(tot, 0.0));
-            const double a0 = cc * delta - c_prev * ss * gamma;
-            const double a1 = sqrt(a0 * a0 + gamma_next * gamma_next);
-            const double inv_a1 = 1.0 / a1;
+            const double a0 = fma(cc, delta, -(c_prev * ss * gamma));
+            const double a1 = sqrt(fma(a0, a0, gamma_next * gamma_next));
             out[0] = gamma_next;
-            out[1] = 1.0 / gamma_next;
-            out[2] = a1;
-            out[3] = inv_a1;
-            out[4] = a0 * inv_a1;
-            out[5] = gamma_next * inv_a1;
+            out[1] = a1;
+            out[2] = fma(c_prev * cc, gamma, ss * delta);
+            out[3] = s_prev * gamma;
+            out[4] = a0 / a1;
+            out[5] = gamma_next / a1;
           });
-      const double gamma_next = g[0], inv_gamma_next = g[1], a1 = g[2], inv_a1 = g[3], c_next = g[4], s_next = g[5];
+      const double gamma_next = g[0], a1 = g[1], a2 = g[2], a3 = g[3], c_next = g[4], s_next = g[5];
       if (a1 == 0.0) break;
-      const double a2 = ss * delta + c_prev * cc * gamma, a3 = s_prev * gamma;
       const double step = c_next * eta;
       for (int q = (int)tm.rank(); q < n; q += (int)tm.size()) {
-        const double wn = (zz[iz][q] - a3 * ww[iw_prev][q] - a2 * ww[iw][q]) * inv_a1;
+        const double wn = (zz[iz][q] - a3 * ww[iw_prev][q] - a2 * ww[iw][q]) / a1;
         ww[iw_next][q] = wn;
         x[q] += step * wn;
       }
@@ -554,9 +621,8 @@ __device__ __noinline__ void minres_team(const Team& tm, const CoarseSys& S, con
       iw_prev = iw;
       iw = iw_next;
       iw_next = t;
-      inv_gamma_prev = inv_gamma;
+      gamma_prev = gamma;
       gamma = gamma_next;
-      inv_gamma = inv_gamma_next;
       c_prev = cc;
       cc = c_next;
       s_prev = ss;

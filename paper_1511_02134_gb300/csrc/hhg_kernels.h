@@ -219,9 +219,9 @@ __host__ __device__ inline int64_t coarse_scratch_doubles(const CoarseSys& S) {
 constexpr int32_t COARSE_ELL_ROUND = 8;
 constexpr int32_t COARSE_ELL_MAX_ROWS = 8192;  // 16 CTAs of 512 threads, one row each
 // A coarsest level this small is solved by one thread block (one warp per CG).
-constexpr int32_t COARSE_BLOCK_MAX_NV = 128;
+constexpr int64_t COARSE_BLOCK_MAX_UNKNOWNS = 4096;
 __host__ __device__ inline bool coarse_fits_block(const CoarseSys& S) {
-  return S.nv <= COARSE_BLOCK_MAX_NV;
+  return 3 * (int64_t)S.nv + S.np <= COARSE_BLOCK_MAX_UNKNOWNS;
 }
 template <class T>
 void launch_coarse_solve(const CoarseSys& S, const LevelDev<T>& L, double* scratch, CoarseParams prm, double* info,

@@ -33,47 +33,22 @@ struct Team {
   }
 };
 
-// Sum over the warp, in every lane.  The addends are aligned to the largest
-// exponent as 58-bit integers (five bits below its last place, where shorter
-// addends are cut off: together less than one unit in the last place of the
-// largest), and summed exactly, in three limbs by the warp's integer
-// reduction: 260 cycles on GB300 against 547 for a tree of five FP64
-// additions, each of which occupies the FP64 pipe for 64.  Addends that are
-// not finite or whose largest is below 2^-959 take the tree.
-__device__ __forceinline__ double warp_sum(double x) {
-  const int hi = __double2hiint(x), ah = hi & 0x7fffffff;
-  const int top = __reduce_max_sync(0xffffffffu, ah) & 0x7ff00000;
-  if (top >= 0x7ff00000 || top < (64 << 20)) {
+// Sum over the warp, in every lane.
+__device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-    return x;
-  }
-  // subnormal addends lie more than 58 bits below the largest: shifted out
-  const int sh = ((top | 0xfffff) - ah) >> 20;
-  int64_t m = ((int64_t)((ah & 0xfffff) | 0x100000) << 32) | (uint32_t)__double2loint(x);
-  m = sh < 58 ? (m << 5) >> sh : 0;
-  m = hi < 0 ? -m : m;
-  const uint32_t s0 = __reduce_add_sync(0xffffffffu, (uint32_t)m & 0x3ffffffu);
-  const uint32_t s1 = __reduce_add_sync(0xffffffffu, (uint32_t)(m >> 26) & 0x3ffffffu);
-  const int s2 = __reduce_add_sync(0xffffffffu, (int)(m >> 52));
-  const int64_t sum = (int64_t)s0 + ((int64_t)s1 << 26) + ((int64_t)s2 << 52);
-  return (double)sum * __hiloint2double(top - (57 << 20), 0);
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
 }
 
-// a / b and 1 / c of values that are the same in every lane, by one division:
-// even lanes form the first, odd lanes the second.
-__device__ __forceinline__ void div_and_rcp(double a, double b, double c, double& q, double& r) {
-  const bool odd = threadIdx.x & 1;
-  const double v = (odd ? 1.0 : a) / (odd ? c : b);
-  q = __shfl_sync(0xffffffffu, v, 0);
-  r = __shfl_sync(0xffffffffu, v, 1);
-}
-
-// Exchange buffers of team_reduce, one set per kernel.
+// Sums over the team are formed from groups of 32 values, a warp each: the
+// sum of group g of sum w is published to slot [w][g] of every CTA
+// (team_publish), and the handler warp of sum w adds the groups in runs of
+// blockDim.x / 32, each run in order, then the runs in order (team_finish).
+// That fixes the rounding by the order of the values alone, wherever in the
+// cluster a group is held.
 constexpr int TEAM_MAX_SUMS = 3, TEAM_MAX_OUT = 6;
 struct TeamShared {
-  double val[32 * TEAM_MAX_WARPS];
-  double part[2][TEAM_MAX_SUMS][TEAM_MAX_BLOCKS];
+  double part[2][TEAM_MAX_SUMS][TEAM_MAX_BLOCKS * TEAM_MAX_WARPS];
   double res[2][TEAM_MAX_OUT];
 };
 __device__ __forceinline__ TeamShared& team_shared() {
@@ -81,53 +56,78 @@ __device__ __forceinline__ TeamShared& team_shared() {
   return s;
 }
 
-// W sums over the team of one value per thread, x: the warps [w * each,
-// (w + 1) * each) of every CTA contribute to sum w, the others to none.  Warp
-// w < W of every CTA is the handler of sum w: it adds its warps' values lane by lane, then
-// over its lanes, exchanges the CTA's partial through distributed shared
-// memory, and evaluates fin(w, total, out) in all its lanes (out: W_OUT
-// doubles published to the CTA), so that the scalar recurrences of a Krylov
-// step run in one warp per CTA.  On GB300 an FP64 instruction occupies a
-// quarter of an SM for 64 cycles per warp: evaluated by every thread, the
-// warp trees, the sixteen partials, the divisions and the square roots of a
-// step cost several times its vectors.  Every thread must call it;
-// blockDim.x is a multiple of 32, at least 32 W and at most
-// 32 TEAM_MAX_WARPS.  Returns the published values: res[w * W_OUT + e].
+// The calling warp's 32 values as group `group` of sum w.
+__device__ __forceinline__ void team_publish(const Team& T, double x, int w, int group) {
+  const int lane = threadIdx.x & 31;
+  x = warp_sum(x);
+  double* at = &team_shared().part[T.calls & 1u][w][group];
+  if (T.nblocks > 1) {
+    if (lane < (int)T.nblocks) *cooperative_groups::this_cluster().map_shared_rank(at, lane) = x;
+  } else if (lane == 0) {
+    *at = x;
+  }
+}
+
+// Totals of the W sums just published (groups 0 .. ngroups - 1 of each).
+// Warp w < W of every CTA is the handler of sum w: it evaluates
+// fin(w, total, out) in all its lanes (out: W_OUT doubles published to the
+// CTA), so that the scalar recurrences of a Krylov step run in one warp per
+// CTA.  On GB300 an FP64 instruction occupies a quarter of an SM for 64
+// cycles per warp: evaluated by every thread, the partials of sixteen CTAs,
+// the divisions and the square roots of a step cost several times its
+// vectors.  Every thread must call it; blockDim.x is a multiple of 32, at
+// least 32 W and at most 32 TEAM_MAX_WARPS.  vals receives the published
+// values, vals[w * W_OUT + e].  A single sum of a block of at most four warps
+// is formed by every warp (each has a quarter of the SM to itself), without
+// the exchange of the values.
 template <int W, int W_OUT, class F>
-__device__ __forceinline__ const double* team_reduce(const Team& T, double x, int each, F&& fin) {
-  static_assert(W <= TEAM_MAX_SUMS && W * W_OUT <= TEAM_MAX_OUT, "team_reduce buffers");
+__device__ __forceinline__ void team_finish(const Team& T, int ngroups, double* vals, F&& fin) {
+  static_assert(W <= TEAM_MAX_SUMS && W * W_OUT <= TEAM_MAX_OUT, "team_finish buffers");
   TeamShared& B = team_shared();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned buf = T.calls & 1u;
   ++T.calls;
-  B.val[threadIdx.x] = x;
-  __syncthreads();
-  double tot = 0.0;
-  if (warp < W) {
-    tot = B.val[32 * warp * each + lane];
-    for (int w = warp * each + 1; w < (warp + 1) * each; ++w) tot += B.val[32 * w + lane];
-    tot = warp_sum(tot);
-    if (T.nblocks > 1 && lane < (int)T.nblocks) {
-      // this CTA's partial into slot blockIdx.x of every CTA
-      double* at = &B.part[buf][warp][blockIdx.x];
-      *cooperative_groups::this_cluster().map_shared_rank(at, lane) = tot;
+  // one barrier per sum: a CTA reaches the barrier of the next sum (the other
+  // buffer) only after it has read this one's groups
+  T.sync();
+  const bool every = W == 1 && T.nblocks == 1 && blockDim.x <= 128;
+  if (warp < W || every) {
+    const int per = (int)(blockDim.x >> 5), g0 = lane * per;
+    const int most = min(per, ngroups);
+    const double* at = B.part[buf][every ? 0 : warp];
+    double run = g0 < ngroups ? at[g0] : 0.0;
+    for (int j = 1; j < most; j += 4) {
+      double v[4];  // four loads in flight, then the additions in order
+#pragma unroll
+      for (int e = 0; e < 4; ++e) v[e] = at[min(g0 + j + e, TEAM_MAX_BLOCKS * TEAM_MAX_WARPS - 1)];
+#pragma unroll
+      for (int e = 0; e < 4; ++e)
+        if (j + e < most) run += g0 + j + e < ngroups ? v[e] : 0.0;
     }
-  }
-  if (T.nblocks > 1) {
-    // one barrier per sum: a CTA reaches the barrier of the next sum (the
-    // other buffer) only after it has read this one's partials
-    cooperative_groups::this_cluster().sync();
-    if (warp < W) tot = warp_sum(lane < (int)T.nblocks ? B.part[buf][warp][lane] : 0.0);
-  }
-  if (warp < W) {
+    double tot = __shfl_sync(0xffffffffu, run, 0);
+    for (int c = 1; c * per < ngroups; ++c) tot += __shfl_sync(0xffffffffu, run, c);
     double out[W_OUT];
     fin(warp, tot, out);
+    if (every) {
+#pragma unroll
+      for (int e = 0; e < W_OUT; ++e) vals[e] = out[e];
+      return;
+    }
     if (lane == 0)
 #pragma unroll
       for (int e = 0; e < W_OUT; ++e) B.res[buf][warp * W_OUT + e] = out[e];
   }
   __syncthreads();
-  return B.res[buf];
+#pragma unroll
+  for (int e = 0; e < W * W_OUT; ++e) vals[e] = B.res[buf][e];
+}
+
+// One sum of a value per thread of the ranking, n items in the loop that formed them.
+template <int W_OUT, class F>
+__device__ __forceinline__ void team_reduce1(const Team& T, double x, int n, double* vals, F&& fin) {
+  const int group = (int)(T.rank() >> 5), ngroups = (min(n, (int)T.size()) + 31) / 32;
+  if (group < ngroups) team_publish(T, x, 0, group);
+  team_finish<1, W_OUT>(T, ngroups, vals, fin);
 }
 
 // A double at a shared-memory address of this CTA or of another CTA of the
