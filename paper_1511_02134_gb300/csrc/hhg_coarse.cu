@@ -20,7 +20,8 @@ template <class T>
 __global__ void __launch_bounds__(CT) k_coarse_minres(CoarseSys S, LevelDev<T> L, double* scratch, CoarseParams prm,
                                                       double* info, unsigned nblocks) {
   pdl_enter();
-  coarse::minres_team(Team{nblocks}, S, L, scratch, prm, info);
+  extern __shared__ __align__(16) double team_mem[];
+  coarse::minres_team(Team{nblocks, team_mem}, S, L, scratch, prm, info);
 }
 
 unsigned g_coarse_cluster = 8;
@@ -44,7 +45,7 @@ void launch_coarse_solve(const CoarseSys& S, const LevelDev<T>& L, double* scrat
                          cudaStream_t s) {
   unsigned nb, th;
   coarse_shape(S, nb, th);
-  launch_team(k_coarse_minres<T>, nb, th, s, S, L, scratch, prm, info, nb);
+  launch_team(k_coarse_minres<T>, nb, th, team_bytes(nb), s, S, L, scratch, prm, info, nb);
 }
 
 template void launch_coarse_solve<double>(const CoarseSys&, const LevelDev<double>&, double*, CoarseParams, double*,
@@ -105,7 +106,7 @@ int coarse_solve_noalloc(const CoarseSys& S, const LevelDev<double>& L, CoarsePa
   }
   unsigned nb, th;
   coarse_shape(S, nb, th);
-  e = launch_team(k_coarse_minres<double>, nb, th, s, S, L, ptr, prm, info, nb);
+  e = launch_team(k_coarse_minres<double>, nb, th, team_bytes(nb), s, S, L, ptr, prm, info, nb);
   if (e == cudaSuccess) e = cudaGetLastError();
   if (e != cudaSuccess) {
     err = std::string("coarse solve launch: ") + cudaGetErrorString(e);

@@ -75,14 +75,14 @@ __device__ inline void applyK(const Ctx& C, const double* x, double* y) {
 // level 1 (1,427 rows, 16 CTAs) an iteration takes 5.5 us, against 27 us
 // with every thread evaluating the scalars and the vectors in global memory.
 constexpr int CG_ROW = COARSE_ELL_ROUND;
-constexpr int CG_DIR = 512;  // directions of a CTA: one per thread
 
 template <int NSYS>
 __device__ __noinline__ int cg_team_regs(const Ctx& C, const double* b, double* x, double* dir, int max_it,
                                          double rtol) {
+  const Team T = C.T;  // local copies: the context is in memory
   const int N = NSYS == 3 ? C.S.nv : 3 * C.S.nv;
   const int groups = (N + 31) / 32;
-  const int each = (groups + (int)C.T.nblocks - 1) / (int)C.T.nblocks;  // groups of a system per CTA
+  const int each = (groups + (int)T.nblocks - 1) / (int)T.nblocks;  // groups of a system per CTA
   const int rc = 32 * each;                                            // its rows
   const int warp = threadIdx.x >> 5, sys = warp / each;
   const bool used = sys < NSYS;
@@ -116,9 +116,9 @@ __device__ __noinline__ int cg_team_regs(const Ctx& C, const double* b, double* 
   double rr = 0.0, stop = 0.0;
   bool run = false;
   int its = 0;
-  if (live) team_publish(C.T, rv * rv, mine, group);
+  if (live) team_publish(T, rv * rv, mine, group);
   double res[2 * NSYS];
-  team_finish<NSYS, 2>(C.T, groups, res, [&](int, double tot, double* out) {
+  team_finish<NSYS, 2>(T, groups, res, [&](int, double tot, double* out) {
     rr = tot;
     stop = rtol * rtol * tot;
     run = !(rr <= stop || rr == 0.0);
@@ -138,7 +138,8 @@ __device__ __noinline__ int cg_team_regs(const Ctx& C, const double* b, double* 
       for (int e = 0; e < CG_ROW; ++e) dn[e] = ld_team_shared(ad[e]);
       qv = 0.0;
 #pragma unroll
-      for (int e = 0; e < CG_ROW; ++e) qv = fma(av[e], dn[e], qv);
+      for (int e = 0; e < CG_ROW; ++e)
+        if (e < len) qv = fma(av[e], dn[e], qv);
       for (int k = CG_ROW; k < len; k += CG_ROW) {
         double a[CG_ROW];
         uint32_t at[CG_ROW];
@@ -154,9 +155,9 @@ __device__ __noinline__ int cg_team_regs(const Ctx& C, const double* b, double* 
           if (k + e < len) qv = fma(a[e], dn[e], qv);
       }
       if (!on) qv = 0.0;
-      team_publish(C.T, dv * qv, mine, group);
+      team_publish(T, dv * qv, mine, group);
     }
-    team_finish<NSYS, 2>(C.T, groups, res, [&](int, double tot, double* out) {
+    team_finish<NSYS, 2>(T, groups, res, [&](int, double tot, double* out) {
       if (run && tot == 0.0) run = false;
       out[0] = run ? 1.0 : 0.0;
       out[1] = run ? rr / tot : 0.0;
@@ -165,10 +166,10 @@ __device__ __noinline__ int cg_team_regs(const Ctx& C, const double* b, double* 
     if (go) {
       const double alpha = res[2 * mine + 1];
       rv = fma(-alpha, qv, rv);
-      team_publish(C.T, rv * rv, mine, group);
+      team_publish(T, rv * rv, mine, group);
       xv = fma(alpha, dv, xv);
     }
-    team_finish<NSYS, 2>(C.T, groups, res, [&](int, double tot, double* out) {
+    team_finish<NSYS, 2>(T, groups, res, [&](int, double tot, double* out) {
       out[0] = out[1] = 0.0;
       if (run) {
         out[1] = tot / rr;
@@ -182,13 +183,14 @@ __device__ __noinline__ int cg_team_regs(const Ctx& C, const double* b, double* 
       dv = fma(res[2 * mine + 1], dv, rv);
       dir[mine * rc + l] = dv;
     }
-    C.T.sync();
+    T.sync();
   }
   if (on) x[idx] = xv;
-  team_finish<NSYS, 1>(C.T, 0, res, [&](int, double, double* out) { out[0] = (double)its; });
+  team_finish<NSYS, 1>(T, 0, res, [&](int, double, double* out) { out[0] = (double)its; });
   double n = 0.0;
 #pragma unroll
   for (int s = 0; s < NSYS; ++s) n += res[s];
+  C.T.calls = T.calls;
   return (int)n;
 }
 
@@ -198,16 +200,19 @@ __device__ __noinline__ int cg_team_regs(const Ctx& C, const double* b, double* 
 template <int NSYS>
 __device__ __noinline__ int cg_team_mem(const Ctx& C, const double* b, double* x, double* cg, int max_it,
                                         double rtol) {
+  const Team T = C.T;  // local copies: the context is in memory
   const int N = NSYS == 3 ? C.S.nv : 3 * C.S.nv;
+  const int32_t *aptr = C.S.aptr, *acol = C.S.acol;
+  const double* aval = C.S.aval;
   double* R = cg;
   double* D = cg + NSYS * N;
   double* Q = cg + 2 * NSYS * N;
-  const int t0 = (int)C.T.rank(), step = (int)C.T.size();
+  const int t0 = (int)T.rank(), step = (int)T.size();
   const int group = t0 >> 5, groups = (min(N, step) + 31) / 32;
   auto publish = [&](const double (&v)[NSYS]) {
     if (group < groups)
 #pragma unroll
-      for (int s = 0; s < NSYS; ++s) team_publish(C.T, v[s], s, group);
+      for (int s = 0; s < NSYS; ++s) team_publish(T, v[s], s, group);
   };
   double acc[NSYS];
 #pragma unroll
@@ -226,7 +231,7 @@ __device__ __noinline__ int cg_team_mem(const Ctx& C, const double* b, double* x
   int its = 0;
   publish(acc);
   double res[2 * NSYS];
-  team_finish<NSYS, 2>(C.T, groups, res, [&](int, double tot, double* out) {
+  team_finish<NSYS, 2>(T, groups, res, [&](int, double tot, double* out) {
     rr = tot;
     stop = rtol * rtol * tot;
     run = !(rr <= stop || rr == 0.0);
@@ -243,13 +248,13 @@ __device__ __noinline__ int cg_team_mem(const Ctx& C, const double* b, double* x
       acc[s] = 0.0;
       if (res[2 * s] == 0.0) continue;
       for (int q = t0; q < N; q += step) {
-        const double aq = csr_row(C.S.aptr, C.S.acol, C.S.aval, q, D + s * N);
+        const double aq = csr_row(aptr, acol, aval, q, D + s * N);
         Q[s * N + q] = aq;
         acc[s] = fma(D[s * N + q], aq, acc[s]);
       }
     }
     publish(acc);
-    team_finish<NSYS, 2>(C.T, groups, res, [&](int, double tot, double* out) {
+    team_finish<NSYS, 2>(T, groups, res, [&](int, double tot, double* out) {
       if (run && tot == 0.0) run = false;
       out[0] = run ? 1.0 : 0.0;
       out[1] = run ? rr / tot : 0.0;
@@ -269,7 +274,7 @@ __device__ __noinline__ int cg_team_mem(const Ctx& C, const double* b, double* x
         }
     }
     publish(acc);
-    team_finish<NSYS, 2>(C.T, groups, res, [&](int, double tot, double* out) {
+    team_finish<NSYS, 2>(T, groups, res, [&](int, double tot, double* out) {
       out[0] = out[1] = 0.0;
       if (run) {
         out[1] = tot / rr;
@@ -285,28 +290,84 @@ __device__ __noinline__ int cg_team_mem(const Ctx& C, const double* b, double* x
         const double beta = res[2 * s + 1];
         for (int q = t0; q < N; q += step) D[s * N + q] = R[s * N + q] + beta * D[s * N + q];
       }
-    C.T.sync();
+    T.sync();
   }
-  team_finish<NSYS, 1>(C.T, 0, res, [&](int, double, double* out) { out[0] = (double)its; });
+  team_finish<NSYS, 1>(T, 0, res, [&](int, double, double* out) { out[0] = (double)its; });
   double n = 0.0;
 #pragma unroll
   for (int s = 0; s < NSYS; ++s) n += res[s];
+  C.T.calls = T.calls;
   return (int)n;
 }
 
 // Team CG of the preconditioner; cg: 9 nv entries of global scratch, dir:
-// CG_DIR entries of shared memory.  One row per lane covers nv <= 2,560 on
-// 16 CTAs of 512 threads.  (One block keeps its few rows in memory, L1: the
-// cube's level 2 in the D form, 81 rows, 355 us per solve against 378.)
+// team_dirs entries of shared memory.  One row per lane covers nv <= 2,560 on
+// 16 CTAs of 512 threads.
 template <int NSYS>
 __device__ inline int cg_team(const Ctx& C, const double* b, double* x, double* cg, double* dir, int max_it,
                               double rtol) {
   const int N = NSYS == 3 ? C.S.nv : 3 * C.S.nv;
   if (N == 0) return 0;  // no velocity unknown (the unit cube's level 0): A has no rows
   const int each = ((N + 31) / 32 + (int)C.T.nblocks - 1) / (int)C.T.nblocks;
-  if (C.T.nblocks > 1 && C.S.eval && 32 * NSYS * each <= min((int)blockDim.x, CG_DIR))
+  if (C.S.eval && 32 * NSYS * each <= min((int)blockDim.x, team_dirs(C.T.nblocks)))
     return cg_team_regs<NSYS>(C, b, x, dir, max_it, rtol);
   return cg_team_mem<NSYS>(C, b, x, cg, max_it, rtol);
+}
+
+// The coupled block on one thread block (few rows: vectors and matrix in
+// L1), every thread evaluating the scalars.  block_sum: the groups of 32
+// values in order, as team_finish forms them.
+__device__ __forceinline__ double block_sum(const Team& T, double x) {
+  double* part = T.part(T.calls & 1u, 0);
+  ++T.calls;
+  x = warp_sum(x);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = x;
+  __syncthreads();
+  double tot = part[0];
+  for (int g = 1; g < (int)(blockDim.x >> 5); ++g) tot += part[g];
+  return tot;
+}
+
+__device__ inline int cg_coupled_block(const Ctx& C, const double* b, double* x, double* cg, int max_it, double rtol) {
+  const int n = 3 * C.S.nv;
+  double* R = cg;
+  double* D = cg + n;
+  double* Q = cg + 2 * n;
+  double rr = 0.0;
+  for (int q = (int)threadIdx.x; q < n; q += (int)blockDim.x) {
+    x[q] = 0.0;
+    R[q] = b[q];
+    D[q] = b[q];
+    rr = fma(b[q], b[q], rr);
+  }
+  rr = block_sum(C.T, rr);
+  const double stop = rtol * rtol * rr;
+  int it = 0;
+  for (; it < max_it; ++it) {
+    if (rr <= stop || rr == 0.0) break;
+    double dq = 0.0;
+    for (int q = (int)threadIdx.x; q < n; q += (int)blockDim.x) {
+      const double aq = csr_row(C.S.aptr, C.S.acol, C.S.aval, q, D);
+      Q[q] = aq;
+      dq = fma(D[q], aq, dq);
+    }
+    dq = block_sum(C.T, dq);
+    if (dq == 0.0) break;
+    const double alpha = rr / dq;
+    double rn = 0.0;
+    for (int q = (int)threadIdx.x; q < n; q += (int)blockDim.x) {
+      x[q] = fma(alpha, D[q], x[q]);
+      const double rq = fma(-alpha, Q[q], R[q]);
+      R[q] = rq;
+      rn = fma(rq, rq, rn);
+    }
+    rn = block_sum(C.T, rn);
+    const double beta = rn / rr;
+    for (int q = (int)threadIdx.x; q < n; q += (int)blockDim.x) D[q] = fma(beta, D[q], R[q]);
+    __syncthreads();
+    rr = rn;
+  }
+  return it;
 }
 
 // ---- warp-level CG: the three velocity blocks are solved concurrently ------
@@ -320,6 +381,8 @@ __device__ inline int cg_team(const Ctx& C, const double* b, double* x, double* 
 template <int NR>
 __device__ __noinline__ int cg_warp(const CoarseSys& S, const double* b, double* x, double* dir, int max_it, double rtol) {
   const int lane = threadIdx.x & 31, nv = S.nv;
+  const double* eval = S.eval;
+  const int32_t* ecol = S.ecol;
   constexpr bool KEEP = NR == 1;
   double xv[NR], rv[NR], dv[NR], qv[NR], av[CG_ROW];
   int at[NR], len[NR], ac[CG_ROW];  // a lane without a row reads row 0 and drops it
@@ -333,8 +396,8 @@ __device__ __noinline__ int cg_warp(const CoarseSys& S, const double* b, double*
     if (KEEP) {
 #pragma unroll
       for (int e = 0; e < CG_ROW; ++e) {
-        av[e] = S.eval[e * nv + at[m]];
-        ac[e] = S.ecol[e * nv + at[m]];
+        av[e] = eval[e * nv + at[m]];
+        ac[e] = ecol[e * nv + at[m]];
       }
     }
     xv[m] = 0.0;
@@ -359,14 +422,14 @@ __device__ __noinline__ int cg_warp(const CoarseSys& S, const double* b, double*
         for (int e = 0; e < CG_ROW; ++e) dn[e] = dir[ac[e]];
 #pragma unroll
         for (int e = 0; e < CG_ROW; ++e)
-          s = fma(av[e], dn[e], s);
+          if (e < len[m]) s = fma(av[e], dn[e], s);
       }
       for (int k = KEEP ? CG_ROW : 0; k < len[m]; k += CG_ROW) {
         double a[CG_ROW], dn[CG_ROW];
 #pragma unroll
         for (int e = 0; e < CG_ROW; ++e) {
-          a[e] = __ldg(S.eval + (k + e) * nv + at[m]);
-          dn[e] = dir[__ldg(S.ecol + (k + e) * nv + at[m])];
+          a[e] = __ldg(eval + (k + e) * nv + at[m]);
+          dn[e] = dir[__ldg(ecol + (k + e) * nv + at[m])];
         }
 #pragma unroll
         for (int e = 0; e < CG_ROW; ++e)
@@ -403,9 +466,11 @@ __device__ __noinline__ int cg_warp(const CoarseSys& S, const double* b, double*
   return it;
 }
 
-// The same for any number of rows per lane, on vectors in memory (r, d, w: nv entries each).
-static __device__ __noinline__ int cg_warp_mem(const CoarseSys& S, const double* b, double* x, double* r, double* d,
-                                        double* w, int max_it, double rtol) {
+// The same for any number of rows per lane, on vectors in memory (r, d, w: nv
+// entries each).  Rows in CSR: side by side (ecol), two at a time, they
+// measured between half and 1.4 times the time, as L1 held them or not.
+__device__ inline int cg_warp_mem(const CoarseSys& S, const double* b, double* x, double* r, double* d, double* w,
+                                  int max_it, double rtol) {
   const int lane = threadIdx.x & 31, nv = S.nv;
   double rr = 0.0;
   for (int q = lane; q < nv; q += 32) {
@@ -422,28 +487,17 @@ static __device__ __noinline__ int cg_warp_mem(const CoarseSys& S, const double*
     if (rr <= stop || rr == 0.0) break;
     double dq = 0.0;
     for (int q = lane; q < nv; q += 32) {
-      const int len = S.aptr[q + 1] - S.aptr[q];
-      double s = 0.0;
-      for (int k = 0; k < len; k += CG_ROW) {
-        double a[CG_ROW], dn[CG_ROW];
-#pragma unroll
-        for (int e = 0; e < CG_ROW; ++e) {
-          a[e] = __ldg(S.eval + (k + e) * nv + q);
-          dn[e] = d[__ldg(S.ecol + (k + e) * nv + q)];
-        }
-#pragma unroll
-        for (int e = 0; e < CG_ROW; ++e) s = fma(a[e], dn[e], s);
-      }
-      w[q] = s;
-      dq = fma(d[q], s, dq);
+      const double aq = csr_row(S.aptr, S.acol, S.aval, q, d);
+      w[q] = aq;
+      dq = fma(d[q], aq, dq);
     }
     dq = warp_sum(dq);
     if (dq == 0.0) break;
     const double alpha = rr / dq;
     double rn = 0.0;
     for (int q = lane; q < nv; q += 32) {
-      x[q] += alpha * d[q];
-      const double rq = r[q] - alpha * w[q];
+      x[q] = fma(alpha, d[q], x[q]);
+      const double rq = fma(-alpha, w[q], r[q]);
       r[q] = rq;
       rn = fma(rq, rq, rn);
     }
@@ -451,7 +505,7 @@ static __device__ __noinline__ int cg_warp_mem(const CoarseSys& S, const double*
     const double beta = rn / rr;
     // every lane has read d (the products above) before any lane rewrites it
     __syncwarp();
-    for (int q = lane; q < nv; q += 32) d[q] = r[q] + beta * d[q];
+    for (int q = lane; q < nv; q += 32) d[q] = fma(beta, d[q], r[q]);
     __syncwarp();
     rr = rn;
   }
@@ -468,8 +522,7 @@ constexpr int WARP_CG_MAX_NV = 1024, WARP_CG_REG_NV = 128;
 // runs them in lockstep (cg_team).  cg holds 9 nv scratch entries.
 __device__ inline int precond(const Ctx& C, const double* v, double* z, double* cg, int cg_max, double cg_rtol) {
   __shared__ int its_sh[3];
-  // search directions: of the three warp CGs, or of this CTA's rows in the team CG
-  __shared__ double dir_sh[CG_DIR];
+  double* dir_sh = C.T.dirs();  // directions of the three warp CGs, or of this CTA's rows in the team CG
   int its = 0;
   const int nv = C.S.nv;
   const int warp = threadIdx.x >> 5;
@@ -480,7 +533,9 @@ __device__ inline int precond(const Ctx& C, const double* v, double* z, double* 
   const int ts = (int)C.T.size() - skip;
   if (t0 >= 0)
     for (int q = t0; q < C.S.np; q += ts) z[3 * nv + q] = v[3 * nv + q] / C.S.mass[q];
-  if (C.S.coupled) {
+  if (C.S.coupled && C.T.nblocks == 1 && blockDim.x <= 128) {
+    its = cg_coupled_block(C, v, z, cg, cg_max, cg_rtol);
+  } else if (C.S.coupled) {
     its = cg_team<1>(C, v, z, cg, dir_sh, cg_max, cg_rtol);
   } else if (par) {
     if (warp < 3) {

@@ -312,6 +312,7 @@ struct ResidentCycle {
   uint32_t wts[RES_MAX_LEVELS + 1];  // byte offset of the level's class table copy
   uint32_t blk[RES_MAX_LEVELS + 1];
   uint32_t zero;
+  uint32_t team;  // byte offset of the coarse solve's team memory (hhg_team.cuh)
   uint32_t smem;
   // Node lists of level q (RES_LISTS of them, list l = 8 kind + 2 colour +
   // boundary, with kind 0 velocity (F_VFREE) / 1 pressure (F_ACT) and

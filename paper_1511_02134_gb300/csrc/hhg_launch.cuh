@@ -7,12 +7,12 @@
 namespace hhg {
 
 template <class... KArgs, class... Args>
-cudaError_t launch_team(void (*kernel)(KArgs...), unsigned nblocks, unsigned threads, cudaStream_t s,
+cudaError_t launch_team(void (*kernel)(KArgs...), unsigned nblocks, unsigned threads, unsigned smem, cudaStream_t s,
                         Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(nblocks, 1, 1);
   cfg.blockDim = dim3(threads, 1, 1);
-  cfg.dynamicSmemBytes = 0;
+  cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

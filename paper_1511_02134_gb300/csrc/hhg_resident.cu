@@ -502,10 +502,10 @@ __device__ void r_coarse(const Res<T>& R) {
   cluster_sync();
   if (coarse_fits_block(S.cs)) {
     if (R.rank == 0) {
-      coarse::minres_team(Team{1}, S.cs, S.lv[0], S.scratch, S.prm, S.info);
+      coarse::minres_team(Team{1, reinterpret_cast<double*>(R.sm + S.team)}, S.cs, S.lv[0], S.scratch, S.prm, S.info);
     }
   } else {
-    coarse::minres_team(Team{S.nblocks}, S.cs, S.lv[0], S.scratch, S.prm, S.info);
+    coarse::minres_team(Team{S.nblocks, reinterpret_cast<double*>(R.sm + S.team)}, S.cs, S.lv[0], S.scratch, S.prm, S.info);
   }
   cluster_sync();
 }
@@ -539,6 +539,8 @@ uint64_t layout_resident(ResidentCycle<T>& S) {
   for (int q = 1; q <= S.nres; ++q) nb = std::max(nb, (unsigned)S.nbq[q]);
   S.nblocks = nb;
   uint64_t off = 0;
+  S.team = 0;  // the coarse solve's sums and directions
+  off = align16(team_bytes(coarse_fits_block(S.cs) ? 1 : nb));
   for (int q = 1; q <= S.nres; ++q) {
     S.tab[q] = (uint32_t)off;
     off = align16(off + sizeof(void*) * RES_TAB_FIELDS * (uint64_t)(S.lv[q].nz + 2));

@@ -116,7 +116,7 @@ __device__ void b_prolong(const Team& tm, const LevelDev<T>& Lf, const LevelDev<
 template <class T>
 __device__ void b_coarse(const Team& tm, const SmallCycle<T>& S) {
   if (tm.nblocks > 1 && coarse_fits_block(S.cs)) {
-    if (blockIdx.x == 0) coarse::minres_team(Team{1}, S.cs, S.lv[0], S.scratch, S.prm, S.info);
+    if (blockIdx.x == 0) coarse::minres_team(Team{1, tm.mem}, S.cs, S.lv[0], S.scratch, S.prm, S.info);
   } else {
     coarse::minres_team(tm, S.cs, S.lv[0], S.scratch, S.prm, S.info);
   }
@@ -126,7 +126,8 @@ __device__ void b_coarse(const Team& tm, const SmallCycle<T>& S) {
 template <class R>
 __global__ void __launch_bounds__(ST) k_small_cycle(SmallCycle<R> S) {
   pdl_enter();
-  const Team tm{S.nblocks};
+  extern __shared__ __align__(16) double team_mem[];
+  const Team tm{S.nblocks, team_mem};
   const int top = S.nlev - 1;
   for (int l = top; l >= 1; --l) {
     for (int s = 0; s < S.nu_pre[l]; ++s) b_uzawa(tm, S.lv[l], S.inv6nuh[l], S.omc[l]);
@@ -144,7 +145,7 @@ __global__ void __launch_bounds__(ST) k_small_cycle(SmallCycle<R> S) {
 
 template <class R>
 void launch_small_cycle(const SmallCycle<R>& S, cudaStream_t s) {
-  launch_team(k_small_cycle<R>, S.nblocks, ST, s, S);
+  launch_team(k_small_cycle<R>, S.nblocks, ST, team_bytes(S.nblocks), s, S);
 }
 
 unsigned prepare_small_cycle() {

@@ -14,9 +14,30 @@ namespace hhg {
 constexpr int TEAM_MAX_WARPS = 16;   // per CTA (512 threads)
 constexpr int TEAM_MAX_BLOCKS = 16;  // CTAs of a cluster
 
+// Shared memory of a team's sums and search directions, in doubles: groups
+// per sum and directions per CTA.  One block needs 3.8 KB, a cluster 16.4 KB;
+// it is dynamic shared memory, because a block's solver lives in what the
+// shared memory leaves of L1 (16 KB more took the solve of 3,000 unknowns
+// from 11 to 18 ms).
+constexpr int TEAM_MAX_SUMS = 3, TEAM_MAX_OUT = 6;
+__host__ __device__ constexpr int team_groups(unsigned nblocks) {
+  return nblocks > 1 ? TEAM_MAX_BLOCKS * TEAM_MAX_WARPS : TEAM_MAX_WARPS;
+}
+__host__ __device__ constexpr int team_dirs(unsigned nblocks) { return nblocks > 1 ? 512 : 384; }
+__host__ __device__ constexpr unsigned team_bytes(unsigned nblocks) {
+  return (unsigned)sizeof(double) * (2 * TEAM_MAX_SUMS * team_groups(nblocks) + team_dirs(nblocks));
+}
+
 struct Team {
   unsigned nblocks;            // CTAs in the cluster; the grid is exactly one cluster
+  double* mem;                 // team_bytes(nblocks) of shared memory (at the same offset in every CTA)
   mutable unsigned calls = 0;  // sums formed so far (the same in every thread): picks the exchange buffer
+
+  // groups of sum w in exchange buffer `buf`; the search directions
+  __device__ __forceinline__ double* part(unsigned buf, int w) const {
+    return mem + (buf * TEAM_MAX_SUMS + w) * team_groups(nblocks);
+  }
+  __device__ __forceinline__ double* dirs() const { return mem + 2 * TEAM_MAX_SUMS * team_groups(nblocks); }
 
   // Consecutive warps of the ranking sit on different CTAs, so that a loop
   // over fewer items than threads loads every SM alike (a ranking CTA by CTA
@@ -46,21 +67,11 @@ __device__ __forceinline__ double warp_sum(double v) {
 // blockDim.x / 32, each run in order, then the runs in order (team_finish).
 // That fixes the rounding by the order of the values alone, wherever in the
 // cluster a group is held.
-constexpr int TEAM_MAX_SUMS = 3, TEAM_MAX_OUT = 6;
-struct TeamShared {
-  double part[2][TEAM_MAX_SUMS][TEAM_MAX_BLOCKS * TEAM_MAX_WARPS];
-  double res[2][TEAM_MAX_OUT];
-};
-__device__ __forceinline__ TeamShared& team_shared() {
-  __shared__ TeamShared s;
-  return s;
-}
-
 // The calling warp's 32 values as group `group` of sum w.
 __device__ __forceinline__ void team_publish(const Team& T, double x, int w, int group) {
   const int lane = threadIdx.x & 31;
   x = warp_sum(x);
-  double* at = &team_shared().part[T.calls & 1u][w][group];
+  double* at = T.part(T.calls & 1u, w) + group;
   if (T.nblocks > 1) {
     if (lane < (int)T.nblocks) *cooperative_groups::this_cluster().map_shared_rank(at, lane) = x;
   } else if (lane == 0) {
@@ -83,7 +94,7 @@ __device__ __forceinline__ void team_publish(const Team& T, double x, int w, int
 template <int W, int W_OUT, class F>
 __device__ __forceinline__ void team_finish(const Team& T, int ngroups, double* vals, F&& fin) {
   static_assert(W <= TEAM_MAX_SUMS && W * W_OUT <= TEAM_MAX_OUT, "team_finish buffers");
-  TeamShared& B = team_shared();
+  __shared__ double res[2][TEAM_MAX_OUT];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const unsigned buf = T.calls & 1u;
   ++T.calls;
@@ -94,12 +105,12 @@ __device__ __forceinline__ void team_finish(const Team& T, int ngroups, double* 
   if (warp < W || every) {
     const int per = (int)(blockDim.x >> 5), g0 = lane * per;
     const int most = min(per, ngroups);
-    const double* at = B.part[buf][every ? 0 : warp];
+    const double* at = T.part(buf, every ? 0 : warp);
     double run = g0 < ngroups ? at[g0] : 0.0;
     for (int j = 1; j < most; j += 4) {
       double v[4];  // four loads in flight, then the additions in order
 #pragma unroll
-      for (int e = 0; e < 4; ++e) v[e] = at[min(g0 + j + e, TEAM_MAX_BLOCKS * TEAM_MAX_WARPS - 1)];
+      for (int e = 0; e < 4; ++e) v[e] = at[min(g0 + j + e, team_groups(T.nblocks) - 1)];
 #pragma unroll
       for (int e = 0; e < 4; ++e)
         if (j + e < most) run += g0 + j + e < ngroups ? v[e] : 0.0;
@@ -115,11 +126,11 @@ __device__ __forceinline__ void team_finish(const Team& T, int ngroups, double* 
     }
     if (lane == 0)
 #pragma unroll
-      for (int e = 0; e < W_OUT; ++e) B.res[buf][warp * W_OUT + e] = out[e];
+      for (int e = 0; e < W_OUT; ++e) res[buf][warp * W_OUT + e] = out[e];
   }
   __syncthreads();
 #pragma unroll
-  for (int e = 0; e < W * W_OUT; ++e) vals[e] = B.res[buf][e];
+  for (int e = 0; e < W * W_OUT; ++e) vals[e] = res[buf][e];
 }
 
 // One sum of a value per thread of the ranking, n items in the loop that formed them.
