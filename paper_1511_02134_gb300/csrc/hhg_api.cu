@@ -42,13 +42,15 @@ struct LevelHost {
   int64_t* d_dir_pad = nullptr;
   double* d_dir_val = nullptr;
   int64_t nirr = 0;                  // F_IRR nodes of the level, (k << 42) | (j << 21) | i
-  int64_t* d_irr = nullptr;
+  int64_t* d_irr = nullptr;          // grouped by colour (LevelView::bnd[1])
+  int64_t* d_virr = nullptr;         // those with a velocity (LevelView::bnd[0])
+  int64_t bnd_at[2][5] = {};
   int32_t* d_list = nullptr;         // node lists of the cluster-resident cycle (ResidentCycle::lists)
   int32_t loff[RES_LISTS + 1] = {};  // their offsets
   double* mem64 = nullptr;
   float* mem32 = nullptr;
-  LevelDev<double> d64{};
-  LevelDev<float> d32{};
+  LevelView<double> d64{};
+  LevelView<float> d32{};
 };
 
 template <class T>
@@ -231,11 +233,11 @@ FxState fx_state(hhg_mesh* M) {
 // ---- enqueue helpers (no synchronisation; graph-capturable) -------------------
 
 template <class T>
-LevelDev<T>& view(hhg_mesh* M, int l);
+LevelView<T>& view(hhg_mesh* M, int l);
 template <>
-LevelDev<double>& view<double>(hhg_mesh* M, int l) { return M->lv[l].d64; }
+LevelView<double>& view<double>(hhg_mesh* M, int l) { return M->lv[l].d64; }
 template <>
-LevelDev<float>& view<float>(hhg_mesh* M, int l) { return M->lv[l].d32; }
+LevelView<float>& view<float>(hhg_mesh* M, int l) { return M->lv[l].d32; }
 
 // Error word of the fused passes (the last slot of the scalar block).
 unsigned* err_word(hhg_mesh* M) { return reinterpret_cast<unsigned*>(M->d_scalars + 15); }
@@ -257,14 +259,14 @@ void enq_pres_sweep(hhg_mesh* M, int l) {
 // B u - g formed at each node.
 template <class T>
 void enq_vel_sweep_f(hhg_mesh* M, int l) {
-  const LevelDev<T>& L = view<T>(M, l);
+  const LevelView<T>& L = view<T>(M, l);
   for (int q = 0; q < 4; ++q) launch_vel_colour_rhs<T>(L, q, M->stream);
   M->launches += 4;
 }
 
 template <class T>
 void enq_pres_sweep_f(hhg_mesh* M, int l) {
-  const LevelDev<T>& L = view<T>(M, l);
+  const LevelView<T>& L = view<T>(M, l);
   for (int q = 0; q < 4; ++q) launch_pres_colour_rhs<T>(L, q, M->stream);
   M->launches += 4;
 }
@@ -292,7 +294,7 @@ void enq_uzawa_fused(hhg_mesh* M, int l, int kind = -1) {
 
 template <class T>
 void enq_uzawa(hhg_mesh* M, int l) {
-  const LevelDev<T>& L = view<T>(M, l);
+  const LevelView<T>& L = view<T>(M, l);
   const bool ru = sizeof(T) != 4;
   if (!ru && M->lv[l].fused) {
     enq_uzawa_fused(M, l);
@@ -732,6 +734,7 @@ void release(hhg_mesh* M) {
     cudaFree(H.d_dir_pad);
     cudaFree(H.d_dir_val);
     cudaFree(H.d_irr);
+    cudaFree(H.d_virr);
     cudaFree(H.mem64);
     cudaFree(H.mem32);
   }
@@ -1017,7 +1020,7 @@ int hhg_create_mesh(const double* V, int64_t nv, const int32_t* T, int64_t nt, c
   // Dirichlet nodes and boundary (F_IRR) nodes of every level (compact lists)
   for (int l = M->coarsest; l <= finest; ++l) {
     LevelHost& H = M->lv[l];
-    std::vector<int64_t> lat, pad, irr;
+    std::vector<int64_t> lat, pad, irr, by_colour[2][4];
     for (int64_t k = 0; k < H.sh.nz; ++k)
       for (int64_t j = 0; j < H.sh.ny; ++j)
         for (int64_t i = 0; i < H.sh.nx; ++i) {
@@ -1027,8 +1030,20 @@ int hhg_create_mesh(const double* V, int64_t nv, const int32_t* T, int64_t nt, c
             lat.push_back(q);
             pad.push_back(pad_index(H.px, H.px * H.py, (int)i, (int)j, (int)k));
           }
-          if (f & F_IRR) irr.push_back((k << 42) | (j << 21) | i);
+          if (f & F_IRR) {
+            const int64_t e = (k << 42) | (j << 21) | i;
+            by_colour[1][(i + j + k) & 3].push_back(e);
+            if (f & F_VFREE) by_colour[0][(i + j + k) & 3].push_back(e);
+          }
         }
+    std::vector<int64_t> virr;
+    for (int kind = 0; kind < 2; ++kind)
+      for (int c = 0; c < 4; ++c) {
+        std::vector<int64_t>& all = kind ? irr : virr;
+        H.bnd_at[kind][c] = (int64_t)all.size();
+        all.insert(all.end(), by_colour[kind][c].begin(), by_colour[kind][c].end());
+        H.bnd_at[kind][c + 1] = (int64_t)all.size();
+      }
     H.ndir = (int64_t)lat.size();
     if (H.ndir) {
       if ((rc = dalloc(M, (void**)&H.d_dir_lat, sizeof(int64_t) * lat.size()))) return bail(rc);
@@ -1045,6 +1060,26 @@ int hhg_create_mesh(const double* V, int64_t nv, const int32_t* T, int64_t nt, c
       M->err = std::string("set-up: ") + cudaGetErrorString(e);
       return bail(HHG_ECUDA);
     }
+    if ((rc = dalloc(M, (void**)&H.d_virr, sizeof(int64_t) * std::max<size_t>(virr.size(), 1)))) return bail(rc);
+    if (!virr.empty() &&
+        (e = cudaMemcpy(H.d_virr, virr.data(), sizeof(int64_t) * virr.size(), cudaMemcpyHostToDevice)) != cudaSuccess) {
+      M->err = std::string("set-up: ") + cudaGetErrorString(e);
+      return bail(HHG_ECUDA);
+    }
+    auto bind_boundary = [&](auto& L) {
+      L.bnd[0] = H.d_virr;
+      L.bnd[1] = H.d_irr;
+      for (int kind = 0; kind < 2; ++kind)
+        for (int c = 0; c < 5; ++c) L.bnd_at[kind][c] = H.bnd_at[kind][c];
+      // on affine lattices every node takes class rows: nothing to keep apart.
+      // The FP32 levels of the speculative form are latency bound, and a
+      // boundary block's extra load (its list entry) costs more there than the
+      // divergence it avoids: FP32 Uzawa step, level 5 27.5 -> 31.3 us, level 6
+      // 39.2 -> 44.8 us, level 7 121 -> 103 us; FP64 level 5 71 -> 50 us.
+      L.split = H.nirr > 0 && 2 * H.nirr < H.n_pres && (sizeof(L.nuh) == 8 || !L.spec);
+    };
+    bind_boundary(H.d64);
+    bind_boundary(H.d32);
   }
   {
     LevelHost& H = M->lv[finest];
@@ -1498,7 +1533,7 @@ int hhg_apply_operator(hhg_mesh* M, int32_t level, const double* u, const double
   if ((rc = dalloc(M, (void**)&tmp, sizeof(double) * 12 * (size_t)H.nalloc))) return rc;
   M->device_bytes -= (int64_t)(sizeof(double) * 12 * (size_t)H.nalloc);
   cudaMemsetAsync(tmp, 0, sizeof(double) * 12 * (size_t)H.nalloc, M->stream);
-  LevelDev<double> L = H.d64;
+  LevelView<double> L = H.d64;
   bind_fields(L, tmp, H.nalloc);
   double* stage = nullptr;
   if ((rc = dalloc(M, (void**)&stage, sizeof(double) * 3 * (size_t)n))) {

@@ -62,6 +62,25 @@ struct LevelDev {
   T* rp;
 };
 
+// A level with its boundary lists, for the launchers (kernels take the
+// LevelDev part: 100 bytes more of parameters cost every launch of a small
+// level 0.3 us).
+template <class T>
+struct LevelView : LevelDev<T> {
+  int split;              // boundary (F_IRR) nodes of the colour and residual kernels in blocks of their own
+  const int64_t* bnd[2];  // lattice coordinates ((k << 42) | (j << 21) | i) of the F_IRR nodes with a velocity
+                          // (0) and of all F_IRR nodes (1), grouped by colour: [bnd_at[.][c], bnd_at[.][c + 1])
+  int64_t bnd_at[2][5];
+};
+
+// The boundary nodes of one launch: lattice coordinates, in the first `rows`
+// rows (or planes) of its blocks.
+struct BoundaryNodes {
+  const int64_t* list;
+  int n;
+  int rows;
+};
+
 // Programmatic dependent launch: every kernel of the library is launched so
 // that the next one may be scheduled while it runs.  A kernel first waits
 // until the grid it depends on has completed and its writes are visible

@@ -22,10 +22,23 @@ template <class T>
 dim3 colour_block(const LevelDev<T>& L) {
   return dim3(CB, 1, L.cbz);
 }
+// Boundary nodes of a colour kernel (LevelView::bnd, list `kind`) in blocks of
+// their own, rows 0 .. by - 1 of the grid's y extent; the planes follow.  In
+// lattice order the two ends of a row put a boundary node into 45 % of the
+// warps of a level-7 pressure colour, and each such warp walked the class
+// rows (110 more loads, 65 multiply-adds) beside the closed form.  Measured:
+// cube level 7 pressure sweep, FP32 63.3 -> 46.1 us, FP64 428 -> 275 us.
 template <class T>
-dim3 colour_grid(const LevelDev<T>& L) {
+dim3 colour_grid(const LevelDev<T>& L, int by) {
   const int64_t slots = (int64_t)L.ny * L.nq;
-  return dim3((unsigned)((slots + CB - 1) / CB), (unsigned)((L.nz + L.cbz - 1) / L.cbz), 1);
+  return dim3((unsigned)((slots + CB - 1) / CB), (unsigned)((L.nz + L.cbz - 1) / L.cbz + by), 1);
+}
+template <class T>
+BoundaryNodes boundary_nodes(const LevelView<T>& L, int kind, int colour, bool split) {
+  if (!split) return BoundaryNodes{nullptr, 0, 0};
+  const int64_t a = L.bnd_at[kind][colour], n = L.bnd_at[kind][colour + 1] - a;
+  const int64_t row = (int64_t)colour_grid(L, 0).x * CB * L.cbz;
+  return BoundaryNodes{L.bnd[kind] + a, (int)n, (int)((n + row - 1) / row)};
 }
 template <class T>
 dim3 full_grid(const LevelDev<T>& L) {
@@ -39,13 +52,25 @@ bool spec_level(const LevelDev<T>& L) {
   return L.spec != 0;
 }
 
-// Colour-kernel node: returns false if outside the lattice.
+// Boundary node of thread t; false past the end.
 template <class T>
-__device__ __forceinline__ bool colour_node(const LevelDev<T>& L, int colour, int& i, int& j, int& k) {
+__device__ __forceinline__ bool boundary_node(const LevelDev<T>& L, const BoundaryNodes& B, int64_t t, Node& n) {
+  if (t >= B.n) return false;
+  const int64_t e = B.list[t];
+  n = node_at(L.px, L.pxy, (int)(e & 0x1fffff), (int)((e >> 21) & 0x1fffff), (int)(e >> 42));
+  return true;
+}
+__device__ __forceinline__ int64_t colour_thread() {
+  return (((int64_t)blockIdx.y * gridDim.x + blockIdx.x) * blockDim.z + threadIdx.z) * CB + threadIdx.x;
+}
+
+// Colour-kernel node (by: the grid's rows of boundary blocks): returns false if outside the lattice.
+template <class T>
+__device__ __forceinline__ bool colour_node(const LevelDev<T>& L, int colour, int by, int& i, int& j, int& k) {
   // slot t of plane k: row j = t / nq, quarter-row slot t - j nq (the rows of
   // a plane packed back to back, so that no warp holds only a row's tail)
   const uint64_t t = (uint64_t)blockIdx.x * CB + threadIdx.x;
-  k = blockIdx.y * blockDim.z + threadIdx.z;
+  k = (blockIdx.y - by) * blockDim.z + threadIdx.z;
   const uint64_t row = L.nq == 1 ? t : __umul64hi(t, L.nq_mul);
   if (row >= (uint64_t)L.ny) return false;
   j = (int)row;
@@ -76,20 +101,31 @@ __global__ void k_vel_rhs(LevelDev<T> L) {
 // Gauss-Seidel update of the velocity nodes of one colour.  SPEC: the
 // speculative node form of small levels (hhg_node_ops.cuh).
 // DF: the velocity block's form (1 D form, 0 Laplace form; hhg_node_ops.cuh).
-template <class T, bool SPEC, int DF>
-__global__ void __launch_bounds__(CB * 4) k_vel_colour(LevelDev<T> L, int colour, T inv6nuh) {
+// SPLIT: boundary nodes in the first B.rows block rows (boundary_nodes).
+template <class T, bool SPEC, int DF, bool SPLIT>
+__global__ void __launch_bounds__(CB * 4) k_vel_colour(LevelDev<T> L, int colour, T inv6nuh, BoundaryNodes B) {
   pdl_enter();
+  if (SPLIT && (int)blockIdx.y < B.rows) {
+    Node n;
+    if (boundary_node(L, B, colour_thread(), n)) node_vel_gs<false, T, DF>(L, n, inv6nuh);
+    return;
+  }
   int i, j, k;
-  if (!colour_node(L, colour, i, j, k)) return;
-  node_vel_gs<SPEC, T, DF>(L, node_at(L.px, L.pxy, i, j, k), inv6nuh);
+  if (!colour_node(L, colour, SPLIT ? B.rows : 0, i, j, k)) return;
+  node_vel_gs<SPEC, T, DF, SPLIT>(L, node_at(L.px, L.pxy, i, j, k), inv6nuh);
 }
 
-template <class T, bool SPEC, int DF>
-__global__ void __launch_bounds__(CB * 4) k_vel_colour_rhs(LevelDev<T> L, int colour, T inv6nuh) {
+template <class T, bool SPEC, int DF, bool SPLIT>
+__global__ void __launch_bounds__(CB * 4) k_vel_colour_rhs(LevelDev<T> L, int colour, T inv6nuh, BoundaryNodes B) {
   pdl_enter();
+  if (SPLIT && (int)blockIdx.y < B.rows) {
+    Node n;
+    if (boundary_node(L, B, colour_thread(), n)) node_vel_gs_rhs<false, T, DF>(L, n, inv6nuh);
+    return;
+  }
   int i, j, k;
-  if (!colour_node(L, colour, i, j, k)) return;
-  node_vel_gs_rhs<SPEC, T, DF>(L, node_at(L.px, L.pxy, i, j, k), inv6nuh);
+  if (!colour_node(L, colour, SPLIT ? B.rows : 0, i, j, k)) return;
+  node_vel_gs_rhs<SPEC, T, DF, SPLIT>(L, node_at(L.px, L.pxy, i, j, k), inv6nuh);
 }
 
 // The last velocity colour of a step (backward colour 0) and the first
@@ -101,25 +137,40 @@ __global__ void __launch_bounds__(CB * 4) k_vel_colour_rhs(LevelDev<T> L, int co
 // the node's own pressure update.  So the sequential order is kept.
 // RU: the velocity right-hand side is read from RU (FP64 path) instead of
 // being formed at the node.
-template <class T, bool RU, bool SPEC, int DF>
-__global__ void __launch_bounds__(CB * 4) k_vel_pres_colour0(LevelDev<T> L, T inv6nuh, T omega_over_6c) {
-  pdl_enter();
-  int i, j, k;
-  if (!colour_node(L, 0, i, j, k)) return;
-  const Node n = node_at(L.px, L.pxy, i, j, k);
+template <class T, bool RU, bool SPEC, int DF, bool REG>
+__device__ __forceinline__ void vel_pres_node(const LevelDev<T>& L, const Node& n, T inv6nuh, T omega_over_6c) {
   if (RU)
-    node_vel_gs<SPEC, T, DF>(L, n, inv6nuh);
+    node_vel_gs<SPEC, T, DF, REG>(L, n, inv6nuh);
   else
-    node_vel_gs_rhs<SPEC, T, DF>(L, n, inv6nuh);
-  node_pres_gs_rhs<SPEC>(L, n, omega_over_6c);
+    node_vel_gs_rhs<SPEC, T, DF, REG>(L, n, inv6nuh);
+  node_pres_gs_rhs<SPEC, T, REG>(L, n, omega_over_6c);
 }
 
-template <class T, bool SPEC>
-__global__ void __launch_bounds__(CB * 4) k_pres_colour_rhs(LevelDev<T> L, int colour, T omega_over_6c) {
+template <class T, bool RU, bool SPEC, int DF, bool SPLIT>
+__global__ void __launch_bounds__(CB * 4) k_vel_pres_colour0(LevelDev<T> L, T inv6nuh, T omega_over_6c, BoundaryNodes B) {
   pdl_enter();
+  if (SPLIT && (int)blockIdx.y < B.rows) {
+    Node n;
+    if (boundary_node(L, B, colour_thread(), n))
+      vel_pres_node<T, RU, false, DF, false>(L, n, inv6nuh, omega_over_6c);
+    return;
+  }
   int i, j, k;
-  if (!colour_node(L, colour, i, j, k)) return;
-  node_pres_gs_rhs<SPEC>(L, node_at(L.px, L.pxy, i, j, k), omega_over_6c);
+  if (!colour_node(L, 0, SPLIT ? B.rows : 0, i, j, k)) return;
+  vel_pres_node<T, RU, SPEC, DF, SPLIT>(L, node_at(L.px, L.pxy, i, j, k), inv6nuh, omega_over_6c);
+}
+
+template <class T, bool SPEC, bool SPLIT>
+__global__ void __launch_bounds__(CB * 4) k_pres_colour_rhs(LevelDev<T> L, int colour, T omega_over_6c, BoundaryNodes B) {
+  pdl_enter();
+  if (SPLIT && (int)blockIdx.y < B.rows) {
+    Node n;
+    if (boundary_node(L, B, colour_thread(), n)) node_pres_gs_rhs<false>(L, n, omega_over_6c);
+    return;
+  }
+  int i, j, k;
+  if (!colour_node(L, colour, SPLIT ? B.rows : 0, i, j, k)) return;
+  node_pres_gs_rhs<SPEC, T, SPLIT>(L, node_at(L.px, L.pxy, i, j, k), omega_over_6c);
 }
 
 // ---- FP32 colour kernels with two nodes per thread -------------------------------
@@ -253,16 +304,28 @@ template <class T>
 __global__ void __launch_bounds__(CB * 4) k_pres_colour(LevelDev<T> L, int colour, T omega_over_6c) {
   pdl_enter();
   int i, j, k;
-  if (!colour_node(L, colour, i, j, k)) return;
+  if (!colour_node(L, colour, 0, i, j, k)) return;
   node_pres_gs(L, node_at(L.px, L.pxy, i, j, k), omega_over_6c);
 }
 
-template <class T, int DF>
-__global__ void k_residual(LevelDev<T> L) {
+// SPLIT: boundary nodes in the first B.rows planes of blocks (FP64 only: cube
+// level 7 596 -> 448 us.  In FP32, 92 -> 80 us there, the compiler then
+// contracts the closed form's products differently, and the level's residual
+// would no longer be bit for bit that of the unsplit kernel.)
+template <class T, int DF, bool SPLIT>
+__global__ void k_residual(LevelDev<T> L, BoundaryNodes B) {
   pdl_enter();
-  int i, j, k;
-  if (!full_node(L, i, j, k)) return;
-  node_residual<T, DF>(L, node_at(L.px, L.pxy, i, j, k));
+  if (SPLIT && (int)blockIdx.z < B.rows) {
+    const int64_t t = (((int64_t)blockIdx.z * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x) * (FX * FY) +
+                      FX * threadIdx.y + threadIdx.x;
+    Node n;
+    if (boundary_node(L, B, t, n)) node_residual<T, DF>(L, n);
+    return;
+  }
+  const int i = blockIdx.x * FX + threadIdx.x, j = blockIdx.y * FY + threadIdx.y;
+  const int k = blockIdx.z - (SPLIT ? B.rows : 0);
+  if (i >= L.nx || j >= L.ny) return;
+  node_residual<T, DF, SPLIT>(L, node_at(L.px, L.pxy, i, j, k));
 }
 
 // The residual of the Laplace form on large levels, four nodes per thread:
@@ -345,6 +408,8 @@ __device__ __forceinline__ QuadField<T> quad_field(const T* x, const QuadRows& q
   return f;
 }
 
+// (Boundary blocks of its own, as in k_residual, cost this kernel 128 registers
+// and spills: level 9 4.42 -> 5.49 ms.)
 template <class T>
 __global__ void __launch_bounds__(FX * FY) k_residual_quad(LevelDev<T> L) {
   pdl_enter();
@@ -1272,21 +1337,27 @@ template <class T>
 void launch_vel_rhs(const LevelDev<T>& L, cudaStream_t s) {
   launch_k(k_vel_rhs<T>, full_grid(L), dim3(FX, FY), s, L);
 }
+// The speculative node form together with boundary blocks exists in FP64 only
+// (FP32 levels of the speculative form are not split).
 template <class T>
-void launch_vel_colour(const LevelDev<T>& L, int colour, cudaStream_t s) {
+constexpr bool SPLIT_SPEC = sizeof(T) == 8;
+
+template <class T>
+void launch_vel_colour(const LevelView<T>& L, int colour, cudaStream_t s) {
   const T inv = (T)(1.0 / (6.0 * (double)L.nuh));
-  const bool sp = spec_level(L), df = L.wt2 != nullptr;
-  if (sp && df)
-    launch_k(k_vel_colour<T, true, 1>, colour_grid(L), colour_block(L), s, L, colour, inv);
-  else if (sp)
-    launch_k(k_vel_colour<T, true, 0>, colour_grid(L), colour_block(L), s, L, colour, inv);
-  else if (df)
-    launch_k(k_vel_colour<T, false, 1>, colour_grid(L), colour_block(L), s, L, colour, inv);
+  const bool sp = spec_level(L);
+  // the D form takes class rows at every node: nothing to split
+  const BoundaryNodes B = boundary_nodes(L, 0, colour, L.split && !L.wt2);
+  auto go = [&](auto kernel) { launch_k(kernel, colour_grid(L, B.rows), colour_block(L), s, L, colour, inv, B); };
+  if (L.wt2)
+    sp ? go(k_vel_colour<T, true, 1, false>) : go(k_vel_colour<T, false, 1, false>);
+  else if (L.split)
+    sp ? go(k_vel_colour<T, SPLIT_SPEC<T>, 0, true>) : go(k_vel_colour<T, false, 0, true>);
   else
-    launch_k(k_vel_colour<T, false, 0>, colour_grid(L), colour_block(L), s, L, colour, inv);
+    sp ? go(k_vel_colour<T, true, 0, false>) : go(k_vel_colour<T, false, 0, false>);
 }
 template <class T>
-void launch_vel_colour_rhs(const LevelDev<T>& L, int colour, cudaStream_t s) {
+void launch_vel_colour_rhs(const LevelView<T>& L, int colour, cudaStream_t s) {
   const T inv = (T)(1.0 / (6.0 * (double)L.nuh));
   if constexpr (std::is_same<T, float>::value) {
     if (L.pairs) {
@@ -1294,18 +1365,18 @@ void launch_vel_colour_rhs(const LevelDev<T>& L, int colour, cudaStream_t s) {
       return;
     }
   }
-  const bool sp = spec_level(L), df = L.wt2 != nullptr;
-  if (sp && df)
-    launch_k(k_vel_colour_rhs<T, true, 1>, colour_grid(L), colour_block(L), s, L, colour, inv);
-  else if (sp)
-    launch_k(k_vel_colour_rhs<T, true, 0>, colour_grid(L), colour_block(L), s, L, colour, inv);
-  else if (df)
-    launch_k(k_vel_colour_rhs<T, false, 1>, colour_grid(L), colour_block(L), s, L, colour, inv);
+  const bool sp = spec_level(L);
+  const BoundaryNodes B = boundary_nodes(L, 0, colour, L.split && !L.wt2);
+  auto go = [&](auto kernel) { launch_k(kernel, colour_grid(L, B.rows), colour_block(L), s, L, colour, inv, B); };
+  if (L.wt2)
+    sp ? go(k_vel_colour_rhs<T, true, 1, false>) : go(k_vel_colour_rhs<T, false, 1, false>);
+  else if (L.split)
+    sp ? go(k_vel_colour_rhs<T, SPLIT_SPEC<T>, 0, true>) : go(k_vel_colour_rhs<T, false, 0, true>);
   else
-    launch_k(k_vel_colour_rhs<T, false, 0>, colour_grid(L), colour_block(L), s, L, colour, inv);
+    sp ? go(k_vel_colour_rhs<T, true, 0, false>) : go(k_vel_colour_rhs<T, false, 0, false>);
 }
 template <class T>
-void launch_vel_pres_colour0(const LevelDev<T>& L, bool ru, cudaStream_t s) {
+void launch_vel_pres_colour0(const LevelView<T>& L, bool ru, cudaStream_t s) {
   const T inv = (T)(1.0 / (6.0 * (double)L.nuh));
   const T w = (T)((double)L.omega / (6.0 * (double)L.c));
   const bool sp = spec_level(L);
@@ -1315,30 +1386,29 @@ void launch_vel_pres_colour0(const LevelDev<T>& L, bool ru, cudaStream_t s) {
       return;
     }
   }
-  auto go = [&](auto kernel) { launch_k(kernel, colour_grid(L), colour_block(L), s, L, inv, w); };
-  if (L.wt2) {
-    if (ru && sp)
-      go(k_vel_pres_colour0<T, true, true, 1>);
-    else if (ru)
-      go(k_vel_pres_colour0<T, true, false, 1>);
-    else if (sp)
-      go(k_vel_pres_colour0<T, false, true, 1>);
+  // (FP32 D form: unsplit, see k_residual; its velocity rows are class rows at every node)
+  const bool split = L.split && (sizeof(T) == 8 || !L.wt2);
+  const BoundaryNodes B = boundary_nodes(L, 1, 0, split);
+  auto go = [&](auto kernel) { launch_k(kernel, colour_grid(L, B.rows), colour_block(L), s, L, inv, w, B); };
+  auto pick = [&](auto df, auto split) {
+    constexpr int DF = decltype(df)::value;
+    constexpr bool SP = decltype(split)::value;
+    constexpr bool SPEC = !SP || SPLIT_SPEC<T>;
+    if (ru)
+      sp ? go(k_vel_pres_colour0<T, true, SPEC, DF, SP>) : go(k_vel_pres_colour0<T, true, false, DF, SP>);
     else
-      go(k_vel_pres_colour0<T, false, false, 1>);
-  } else {
-    if (ru && sp)
-      go(k_vel_pres_colour0<T, true, true, 0>);
-    else if (ru)
-      go(k_vel_pres_colour0<T, true, false, 0>);
-    else if (sp)
-      go(k_vel_pres_colour0<T, false, true, 0>);
-    else
-      go(k_vel_pres_colour0<T, false, false, 0>);
-  }
+      sp ? go(k_vel_pres_colour0<T, false, SPEC, DF, SP>) : go(k_vel_pres_colour0<T, false, false, DF, SP>);
+  };
+  using I0 = std::integral_constant<int, 0>;
+  using I1 = std::integral_constant<int, 1>;
+  if (L.wt2)
+    split ? pick(I1(), std::integral_constant<bool, sizeof(T) == 8>()) : pick(I1(), std::false_type());
+  else
+    split ? pick(I0(), std::true_type()) : pick(I0(), std::false_type());
 }
 
 template <class T>
-void launch_pres_colour_rhs(const LevelDev<T>& L, int colour, cudaStream_t s) {
+void launch_pres_colour_rhs(const LevelView<T>& L, int colour, cudaStream_t s) {
   const T w = (T)((double)L.omega / (6.0 * (double)L.c));
   if constexpr (std::is_same<T, float>::value) {
     if (L.pairs) {
@@ -1346,10 +1416,13 @@ void launch_pres_colour_rhs(const LevelDev<T>& L, int colour, cudaStream_t s) {
       return;
     }
   }
-  if (spec_level(L))
-    launch_k(k_pres_colour_rhs<T, true>, colour_grid(L), colour_block(L), s, L, colour, w);
+  const bool sp = spec_level(L);
+  const BoundaryNodes B = boundary_nodes(L, 1, colour, L.split);
+  auto go = [&](auto kernel) { launch_k(kernel, colour_grid(L, B.rows), colour_block(L), s, L, colour, w, B); };
+  if (L.split)
+    sp ? go(k_pres_colour_rhs<T, SPLIT_SPEC<T>, true>) : go(k_pres_colour_rhs<T, false, true>);
   else
-    launch_k(k_pres_colour_rhs<T, false>, colour_grid(L), colour_block(L), s, L, colour, w);
+    sp ? go(k_pres_colour_rhs<T, true, false>) : go(k_pres_colour_rhs<T, false, false>);
 }
 template <class T>
 void launch_pres_rhs(const LevelDev<T>& L, cudaStream_t s) {
@@ -1358,18 +1431,29 @@ void launch_pres_rhs(const LevelDev<T>& L, cudaStream_t s) {
 template <class T>
 void launch_pres_colour(const LevelDev<T>& L, int colour, cudaStream_t s) {
   const T w = (T)((double)L.omega / (6.0 * (double)L.c));
-  launch_k(k_pres_colour<T>, colour_grid(L), colour_block(L), s, L, colour, w);
+  launch_k(k_pres_colour<T>, colour_grid(L, 0), colour_block(L), s, L, colour, w);
 }
 template <class T>
-void launch_residual(const LevelDev<T>& L, cudaStream_t s) {
-  if (L.wt2) {
-    launch_k(k_residual<T, 1>, full_grid(L), dim3(FX, FY), s, L);
-  } else if (L.quad) {
+void launch_residual(const LevelView<T>& L, cudaStream_t s) {
+  if (!L.wt2 && L.quad) {
     const int npos = L.nx / 4 + 1;  // quads cover padded x = 0 .. 4 npos - 1 >= nx
     launch_k(k_residual_quad<T>, dim3((npos + FX - 1) / FX, (L.ny + FY - 1) / FY, L.nz), dim3(FX, FY), s, L);
-  } else {
-    launch_k(k_residual<T, 0>, full_grid(L), dim3(FX, FY), s, L);
+    return;
   }
+  dim3 grid = full_grid(L);
+  constexpr bool SP = sizeof(T) == 8;
+  const bool split = SP && L.split;
+  BoundaryNodes B{nullptr, 0, 0};
+  if (split) {
+    const int64_t n = L.bnd_at[1][4], plane = (int64_t)grid.x * grid.y * (FX * FY);
+    B = BoundaryNodes{L.bnd[1], (int)n, (int)((n + plane - 1) / plane)};
+    grid.z += B.rows;
+  }
+  auto go = [&](auto kernel) { launch_k(kernel, grid, dim3(FX, FY), s, L, B); };
+  if (L.wt2)
+    split ? go(k_residual<T, 1, SP>) : go(k_residual<T, 1, false>);
+  else
+    split ? go(k_residual<T, 0, SP>) : go(k_residual<T, 0, false>);
 }
 template <class T>
 void launch_restrict(const LevelDev<T>& fine, const LevelDev<T>& coarse, cudaStream_t s) {
@@ -1513,13 +1597,13 @@ void launch_cast_field(const double* src, float* dst, int64_t n, cudaStream_t s)
 
 #define HHG_INST(T)                                                                                    \
   template void launch_vel_rhs<T>(const LevelDev<T>&, cudaStream_t);                                    \
-  template void launch_vel_colour<T>(const LevelDev<T>&, int, cudaStream_t);                            \
+  template void launch_vel_colour<T>(const LevelView<T>&, int, cudaStream_t);                            \
   template void launch_pres_rhs<T>(const LevelDev<T>&, cudaStream_t);                                   \
-  template void launch_vel_colour_rhs<T>(const LevelDev<T>&, int, cudaStream_t);                        \
-  template void launch_pres_colour_rhs<T>(const LevelDev<T>&, int, cudaStream_t);                       \
-  template void launch_vel_pres_colour0<T>(const LevelDev<T>&, bool, cudaStream_t);                      \
+  template void launch_vel_colour_rhs<T>(const LevelView<T>&, int, cudaStream_t);                        \
+  template void launch_pres_colour_rhs<T>(const LevelView<T>&, int, cudaStream_t);                       \
+  template void launch_vel_pres_colour0<T>(const LevelView<T>&, bool, cudaStream_t);                      \
   template void launch_pres_colour<T>(const LevelDev<T>&, int, cudaStream_t);                           \
-  template void launch_residual<T>(const LevelDev<T>&, cudaStream_t);                                   \
+  template void launch_residual<T>(const LevelView<T>&, cudaStream_t);                                   \
   template void launch_restrict<T>(const LevelDev<T>&, const LevelDev<T>&, cudaStream_t);               \
   template void launch_prolong_add<T>(const LevelDev<T>&, const LevelDev<T>&, cudaStream_t);            \
   template void launch_residual_norm2<T>(const LevelDev<T>&, double*, double*, cudaStream_t);           \

@@ -12,16 +12,16 @@ namespace hhg {
 
 // Smoother pieces (Sec. 3.3 inexact Uzawa step, Sec. 3.5 smoothers)
 template <class T> void launch_vel_rhs(const LevelDev<T>& L, cudaStream_t s);
-template <class T> void launch_vel_colour(const LevelDev<T>& L, int colour, cudaStream_t s);
+template <class T> void launch_vel_colour(const LevelView<T>& L, int colour, cudaStream_t s);
 template <class T> void launch_pres_rhs(const LevelDev<T>& L, cudaStream_t s);
 template <class T> void launch_pres_colour(const LevelDev<T>& L, int colour, cudaStream_t s);
 // Colour sweeps that form their right-hand side at each node (f - B^T p for
 // velocity, B u - g for pressure) instead of reading RU / RP.
-template <class T> void launch_vel_colour_rhs(const LevelDev<T>& L, int colour, cudaStream_t s);
-template <class T> void launch_pres_colour_rhs(const LevelDev<T>& L, int colour, cudaStream_t s);
+template <class T> void launch_vel_colour_rhs(const LevelView<T>& L, int colour, cudaStream_t s);
+template <class T> void launch_pres_colour_rhs(const LevelView<T>& L, int colour, cudaStream_t s);
 // Backward velocity colour 0 and pressure colour 0 in one launch (the
 // velocity right-hand side read from RU when ru, else formed at the node).
-template <class T> void launch_vel_pres_colour0(const LevelDev<T>& L, bool ru, cudaStream_t s);
+template <class T> void launch_vel_pres_colour0(const LevelView<T>& L, bool ru, cudaStream_t s);
 // Colour-fused FP32 Uzawa step (hhg_fused.cu): three passes over a level,
 // each a z-march of CTAs over (x, y) tiles with F colour phases per march
 // step on planes staged into a shared-memory ring by tensor copies:
@@ -75,7 +75,7 @@ void prepare_fused();
 // 28.2 us, level 6 60 -> 49 us, while level 7 went 170 -> 191 us.
 constexpr int64_t SPEC_MAX_NODES = 1 << 20;
 // Residual (RU, RP) = (F, G) - K (U, P); zero on nodes without unknowns.
-template <class T> void launch_residual(const LevelDev<T>& L, cudaStream_t s);
+template <class T> void launch_residual(const LevelView<T>& L, cudaStream_t s);
 
 // Transfers between level l (fine) and l-1 (coarse).
 template <class T> void launch_restrict(const LevelDev<T>& fine, const LevelDev<T>& coarse, cudaStream_t s);

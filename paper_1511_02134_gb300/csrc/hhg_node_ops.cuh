@@ -40,10 +40,13 @@ __device__ __forceinline__ void node_vel_rhs(const LevelDev<T>& L, const Node& n
 
 // u_d <- u_d + (RU_d - (A u_d)) / A_ii  (one node of the current colour);
 // in the D form the node's three components at once with its 3 x 3 block.
-template <bool SPEC, class T, class V, int DF = -1>
+// REG (here and below): boundary nodes are left out (the kernel updates them
+// in blocks of their own).
+template <bool SPEC, class T, class V, int DF = -1, bool REG = false>
 __device__ __forceinline__ void node_vel_gs_v(const LevelDev<T>& L, int64_t c, const V* u, T inv6nuh) {
   if (d_form<DF>(L)) {
-    if (!(L.flags[c] & F_VFREE)) return;
+    const uint8_t fd = L.flags[c];
+    if (!(fd & F_VFREE) || (REG && (fd & F_IRR))) return;
     const T r[3] = {L.r[0][c], L.r[1][c], L.r[2][c]};
     T out[3];
     vel_block_value(L, d_row(L, c), r, u, out);
@@ -71,6 +74,7 @@ __device__ __forceinline__ void node_vel_gs_v(const LevelDev<T>& L, int64_t c, c
     for (int d = 0; d < 3; ++d) L.u[d][c] = reg[d];
     return;
   }
+  if (REG) return;
   const T* w = class_row(L, c);
   T out[3];
 #pragma unroll
@@ -84,10 +88,10 @@ __device__ __forceinline__ void node_vel_gs_v(const LevelDev<T>& L, int64_t c, c
   for (int d = 0; d < 3; ++d) L.u[d][c] = out[d];
 }
 
-template <bool SPEC, class T, int DF = -1>
+template <bool SPEC, class T, int DF = -1, bool REG = false>
 __device__ __forceinline__ void node_vel_gs(const LevelDev<T>& L, const Node& n, T inv6nuh) {
   const GNb<T> u[3] = {gnb(L.u[0], n, L.px, L.pxy), gnb(L.u[1], n, L.px, L.pxy), gnb(L.u[2], n, L.px, L.pxy)};
-  node_vel_gs_v<SPEC, T, GNb<T>, DF>(L, n.c, u, inv6nuh);
+  node_vel_gs_v<SPEC, T, GNb<T>, DF, REG>(L, n.c, u, inv6nuh);
 }
 
 // New velocity of a regular node from its right-hand side f (3 values) and
@@ -151,12 +155,12 @@ __device__ __forceinline__ void vel_rhs_irr(const LevelDev<T>& L, int64_t c, con
 
 // Same update with the right-hand side f - B^T p formed at the node (p does
 // not change during the velocity sweeps, Sec. 3.3), RU is not touched.
-template <bool SPEC, class T, class V, int DF = -1>
+template <bool SPEC, class T, class V, int DF = -1, bool REG = false>
 __device__ __forceinline__ void node_vel_gs_rhs_v(const LevelDev<T>& L, int64_t c, const V* u, const V& p,
                                                   T inv6nuh) {
   if (d_form<DF>(L)) {
     const uint8_t fl = L.flags[c];
-    if (!(fl & F_VFREE)) return;
+    if (!(fl & F_VFREE) || (REG && (fl & F_IRR))) return;
     T bt[3];
     row_BT_v(L, p, row_of(L, c, fl), fl, bt);
     const T r[3] = {L.f[0][c] - bt[0], L.f[1][c] - bt[1], L.f[2][c] - bt[2]};
@@ -182,13 +186,13 @@ __device__ __forceinline__ void node_vel_gs_rhs_v(const LevelDev<T>& L, int64_t 
     for (int d = 0; d < 3; ++d) L.u[d][c] = reg[d];
     return;
   }
-  vel_rhs_irr(L, c, u, p);
+  if (!REG) vel_rhs_irr(L, c, u, p);
 }
 
-template <bool SPEC, class T, int DF = -1>
+template <bool SPEC, class T, int DF = -1, bool REG = false>
 __device__ __forceinline__ void node_vel_gs_rhs(const LevelDev<T>& L, const Node& n, T inv6nuh) {
   const GNb<T> u[3] = {gnb(L.u[0], n, L.px, L.pxy), gnb(L.u[1], n, L.px, L.pxy), gnb(L.u[2], n, L.px, L.pxy)};
-  node_vel_gs_rhs_v<SPEC, T, GNb<T>, DF>(L, n.c, u, gnb(L.p, n, L.px, L.pxy), inv6nuh);
+  node_vel_gs_rhs_v<SPEC, T, GNb<T>, DF, REG>(L, n.c, u, gnb(L.p, n, L.px, L.pxy), inv6nuh);
 }
 
 // RP = B U - G (pressure nodes).
@@ -257,7 +261,7 @@ __device__ __forceinline__ void pres_rhs_irr(const LevelDev<T>& L, int64_t c, co
 
 // Same update with B u - g formed at the node (u does not change during the
 // pressure sweep), RP is not touched.
-template <bool SPEC, class T, class V>
+template <bool SPEC, class T, class V, bool REG = false>
 __device__ __forceinline__ void node_pres_gs_rhs_v(const LevelDev<T>& L, int64_t c, const V* u, const V& p,
                                                    T omega_over_6c) {
   T reg = (T)0, pc;
@@ -277,20 +281,22 @@ __device__ __forceinline__ void node_pres_gs_rhs_v(const LevelDev<T>& L, int64_t
     L.p[c] = reg;
     return;
   }
-  pres_rhs_irr(L, c, u, p, pc);
+  if (!REG) pres_rhs_irr(L, c, u, p, pc);
 }
 
-template <bool SPEC, class T>
+template <bool SPEC, class T, bool REG = false>
 __device__ __forceinline__ void node_pres_gs_rhs(const LevelDev<T>& L, const Node& n, T omega_over_6c) {
   const GNb<T> u[3] = {gnb(L.u[0], n, L.px, L.pxy), gnb(L.u[1], n, L.px, L.pxy), gnb(L.u[2], n, L.px, L.pxy)};
-  node_pres_gs_rhs_v<SPEC>(L, n.c, u, gnb(L.p, n, L.px, L.pxy), omega_over_6c);
+  node_pres_gs_rhs_v<SPEC, T, GNb<T>, REG>(L, n.c, u, gnb(L.p, n, L.px, L.pxy), omega_over_6c);
 }
 
 // (RU, RP) = (F, G) - K (U, P) at one node, returned in r[0..3]; zero for
 // unknowns the node does not carry.
-template <class T, class V, int DF = -1>
+// REG: the caller knows the node is not a boundary node.
+template <class T, class V, int DF = -1, bool REG = false>
 __device__ __forceinline__ void node_residual_v(const LevelDev<T>& L, int64_t c, uint8_t fl, const V* u, const V& p,
                                                 T r[4]) {
+  if (REG) fl &= (uint8_t)~(F_IRR | F_SLIP);
   const T* w = row_of(L, c, fl);
   if (fl & F_VFREE) {
     T au[3], bt[3];
@@ -309,13 +315,14 @@ __device__ __forceinline__ void node_residual_v(const LevelDev<T>& L, int64_t c,
   r[3] = (fl & F_ACT) ? L.g[c] - row_B_v(L, u, w, fl) + row_C_v(L, p, w, fl) : (T)0;
 }
 
-template <class T, int DF = -1>
+template <class T, int DF = -1, bool REG = false>
 __device__ __forceinline__ void node_residual(const LevelDev<T>& L, const Node& n) {
   const int64_t c = n.c;
   const uint8_t fl = L.flags[c];
+  if (REG && (fl & F_IRR)) return;
   const GNb<T> u[3] = {gnb(L.u[0], n, L.px, L.pxy), gnb(L.u[1], n, L.px, L.pxy), gnb(L.u[2], n, L.px, L.pxy)};
   T r[4];
-  node_residual_v<T, GNb<T>, DF>(L, c, fl, u, gnb(L.p, n, L.px, L.pxy), r);
+  node_residual_v<T, GNb<T>, DF, REG>(L, c, fl, u, gnb(L.p, n, L.px, L.pxy), r);
 #pragma unroll
   for (int d = 0; d < 3; ++d) L.r[d][c] = r[d];
   L.rp[c] = r[3];
