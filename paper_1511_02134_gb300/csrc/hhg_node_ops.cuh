@@ -3,9 +3,42 @@
 // loops over the nodes of a level inside one thread block.  Both call these
 // functions, so the two paths do the same arithmetic in the same order.
 #pragma once
+#include <type_traits>
+
+#include "hhg_aligned.cuh"
 #include "hhg_device.cuh"
 
 namespace hhg {
+
+// Closed-form stencils of regular nodes on one field: FP32 as plain sums, FP64
+// in global memory in aligned integers (hhg_aligned.cuh).  The cluster-resident
+// levels keep the FP64 sums: their phases are latency bound, with fewer warps
+// than FP64 pipes would need to be busy, and the integers spill (cube level 4
+// FP64 solve 8.50 -> 8.60 ms).
+template <class V>
+constexpr bool ALIGNED = std::is_same<V, GNb<double>>::value;
+
+template <class T, class V>
+__device__ __forceinline__ T st_nb6(const V& x) {
+  if constexpr (ALIGNED<V>)
+    return al_nb6(x);
+  else
+    return nb6v(x);
+}
+template <class T, class V>
+__device__ __forceinline__ void st_div12_all(const V& x, T out[3]) {
+  if constexpr (ALIGNED<V>)
+    al_div12_all(x, out);
+  else
+    div12_all(diff7v<T>(x), out);
+}
+template <class T, class V>
+__device__ __forceinline__ T st_div12(const V& x, int comp) {
+  if constexpr (ALIGNED<V>)
+    return al_div12(x, comp);
+  else
+    return div12(diff7v<T>(x), comp);
+}
 
 // Velocity block of the level: DF = 1 the D form (coupled 3 x 3 node blocks),
 // 0 the Laplace form, -1 read from the level (L.wt2 set in the D form).  The
@@ -23,7 +56,14 @@ __device__ __forceinline__ void node_vel_rhs(const LevelDev<T>& L, const Node& n
   const uint8_t fl = L.flags[c];
   if (!(fl & F_VFREE)) return;
   T bt[3];
-  row_BT(L, L.p, n, fl, bt);
+  if (!(fl & F_IRR)) {
+    st_div12_all<T>(gnb(L.p, n, L.px, L.pxy), bt);
+    const T s = -L.h2 * (T)(1.0 / 12.0);
+#pragma unroll
+    for (int d = 0; d < 3; ++d) bt[d] = s * bt[d];
+  } else {
+    row_BT(L, L.p, n, fl, bt);
+  }
 #pragma unroll
   for (int d = 0; d < 3; ++d) L.r[d][c] = L.f[d][c] - bt[d];
 }
@@ -58,7 +98,7 @@ __device__ __forceinline__ void node_vel_gs_v(const LevelDev<T>& L, int64_t c, c
   uint8_t fl;
   if (SPEC) {
 #pragma unroll
-    for (int d = 0; d < 3; ++d) reg[d] = (L.r[d][c] + L.nuh * nb6v(u[d])) * inv6nuh;
+    for (int d = 0; d < 3; ++d) reg[d] = (L.r[d][c] + L.nuh * st_nb6<T>(u[d])) * inv6nuh;
     fl = L.flags[c];
     if (!(fl & F_VFREE)) return;
   } else {
@@ -66,7 +106,7 @@ __device__ __forceinline__ void node_vel_gs_v(const LevelDev<T>& L, int64_t c, c
     if (!(fl & F_VFREE)) return;
     if (!(fl & F_IRR)) {
 #pragma unroll
-      for (int d = 0; d < 3; ++d) reg[d] = (L.r[d][c] + L.nuh * nb6v(u[d])) * inv6nuh;
+      for (int d = 0; d < 3; ++d) reg[d] = (L.r[d][c] + L.nuh * st_nb6<T>(u[d])) * inv6nuh;
     }
   }
   if (!(fl & F_IRR)) {
@@ -129,10 +169,10 @@ template <class T, class V>
 __device__ __forceinline__ void vel_rhs_regular(const LevelDev<T>& L, int64_t c, const V* u, const V& p, T inv6nuh,
                                                 T reg[3]) {
   T dv[3];
-  div12_all(diff7v<T>(p), dv);
+  st_div12_all<T>(p, dv);
   const T s = -L.h2 * (T)(1.0 / 12.0);
 #pragma unroll
-  for (int d = 0; d < 3; ++d) reg[d] = ((L.f[d][c] - s * dv[d]) + L.nuh * nb6v(u[d])) * inv6nuh;
+  for (int d = 0; d < 3; ++d) reg[d] = ((L.f[d][c] - s * dv[d]) + L.nuh * st_nb6<T>(u[d])) * inv6nuh;
 }
 
 // Velocity update of a boundary node (class rows) with f - B^T p formed at
@@ -213,7 +253,7 @@ __device__ __forceinline__ void node_pres_gs(const LevelDev<T>& L, const Node& n
   if (!(fl & F_ACT)) return;
   const T pc = L.p[c];
   if (!(fl & F_IRR)) {
-    const T cp = L.c * ((T)6 * pc - nb6(L.p, n, L.px, L.pxy));
+    const T cp = L.c * ((T)6 * pc - st_nb6<T>(gnb(L.p, n, L.px, L.pxy)));
     L.p[c] = pc + omega_over_6c * (L.rp[c] - cp);
   } else {
     T dg, of;
@@ -228,11 +268,16 @@ __device__ __forceinline__ void node_pres_gs(const LevelDev<T>& L, const Node& n
 template <class T, class V>
 __device__ __forceinline__ T pres_regular_value(const LevelDev<T>& L, T g, const V* u, const V& p, T pc,
                                                 T omega_over_6c) {
-  const T d0 = div12(diff7v<T>(u[0]), 0);
-  const T d1 = div12(diff7v<T>(u[1]), 1);
-  const T d2 = div12(diff7v<T>(u[2]), 2);
+  const T d0 = st_div12<T>(u[0], 0);
+  const T d1 = st_div12<T>(u[1], 1);
+  const T d2 = st_div12<T>(u[2], 2);
   const T rp = L.h2 * (T)(1.0 / 12.0) * ((d0 + d1) + d2) - g;
-  const T cp = L.c * ((T)6 * pc - nb6v(p));
+  T lap;
+  if constexpr (ALIGNED<V>)
+    lap = al_lap7(p);
+  else
+    lap = (T)6 * pc - nb6v(p);
+  const T cp = L.c * lap;
   return pc + omega_over_6c * (rp - cp);
 }
 
@@ -297,6 +342,21 @@ template <class T, class V, int DF = -1, bool REG = false>
 __device__ __forceinline__ void node_residual_v(const LevelDev<T>& L, int64_t c, uint8_t fl, const V* u, const V& p,
                                                 T r[4]) {
   if (REG) fl &= (uint8_t)~(F_IRR | F_SLIP);
+  if constexpr (ALIGNED<V> && DF == 0) {
+    if (!(fl & F_IRR)) {
+      // each field aligned once for its Laplacian and its divergence part
+      T au[3], bu[3], bt[3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) au[d] = al_lap_div(u[d], d, bu + d);
+      const T cp = al_lap_div(p, -1, bt);
+      const T s = L.h2 * (T)(1.0 / 12.0);
+      const bool vf = fl & F_VFREE;
+#pragma unroll
+      for (int d = 0; d < 3; ++d) r[d] = vf ? L.f[d][c] - L.nuh * au[d] + s * bt[d] : (T)0;
+      r[3] = (fl & F_ACT) ? L.g[c] - s * ((bu[0] + bu[1]) + bu[2]) + L.c * cp : (T)0;
+      return;
+    }
+  }
   const T* w = row_of(L, c, fl);
   if (fl & F_VFREE) {
     T au[3], bt[3];
