@@ -22,17 +22,18 @@ template <class T>
 dim3 colour_block(const LevelDev<T>& L) {
   return dim3(CB, 1, L.cbz);
 }
-// Boundary nodes of a colour kernel (LevelView::bnd, list `kind`) in blocks of
-// their own, rows 0 .. by - 1 of the grid's y extent; the planes follow.  In
-// lattice order the two ends of a row put a boundary node into 45 % of the
-// warps of a level-7 pressure colour, and each such warp walked the class
-// rows (110 more loads, 65 multiply-adds) beside the closed form.  Measured:
-// cube level 7 pressure sweep, FP32 63.3 -> 46.1 us, FP64 428 -> 275 us.
 template <class T>
 dim3 colour_grid(const LevelDev<T>& L, int by) {
   const int64_t slots = (int64_t)L.ny * L.nq;
   return dim3((unsigned)((slots + CB - 1) / CB), (unsigned)((L.nz + L.cbz - 1) / L.cbz + by), 1);
 }
+// Boundary nodes of a colour kernel (LevelView::bnd, list `kind`) in blocks of
+// their own, rows 0 .. rows - 1 of the grid's y extent; the planes follow.  In
+// lattice order the two ends of a row put a boundary node into 45 % of the
+// warps of a level-7 pressure colour, and each such warp walked the class
+// rows (110 more loads, 65 multiply-adds) beside the closed form.  Measured:
+// cube level 7 pressure sweep, FP32 62.2 -> 46.1 us, FP64 428 -> 275 us (134
+// with the closed form in aligned integers, hhg_aligned.cuh).
 template <class T>
 BoundaryNodes boundary_nodes(const LevelView<T>& L, int kind, int colour, bool split) {
   if (!split) return BoundaryNodes{nullptr, 0, 0};
@@ -309,7 +310,7 @@ __global__ void __launch_bounds__(CB * 4) k_pres_colour(LevelDev<T> L, int colou
 }
 
 // SPLIT: boundary nodes in the first B.rows planes of blocks (FP64 only: cube
-// level 7 596 -> 448 us.  In FP32, 92 -> 80 us there, the compiler then
+// level 7 596 -> 448 us, 215 with aligned integers.  In FP32, 92 -> 80 us there, the compiler then
 // contracts the closed form's products differently, and the level's residual
 // would no longer be bit for bit that of the unsplit kernel.)
 template <class T, int DF, bool SPLIT>
