@@ -32,7 +32,7 @@ dim3 colour_grid(const LevelDev<T>& L, int by) {
 // lattice order the two ends of a row put a boundary node into 45 % of the
 // warps of a level-7 pressure colour, and each such warp walked the class
 // rows (110 more loads, 65 multiply-adds) beside the closed form.  Measured:
-// cube level 7 pressure sweep, FP32 62.2 -> 46.1 us, FP64 428 -> 275 us (134
+// cube level 7 pressure sweep, FP32 62.2 -> 46.1 us, FP64 428 -> 275 us (144
 // with the closed form in aligned integers, hhg_aligned.cuh).
 template <class T>
 BoundaryNodes boundary_nodes(const LevelView<T>& L, int kind, int colour, bool split) {
@@ -310,7 +310,7 @@ __global__ void __launch_bounds__(CB * 4) k_pres_colour(LevelDev<T> L, int colou
 }
 
 // SPLIT: boundary nodes in the first B.rows planes of blocks (FP64 only: cube
-// level 7 596 -> 448 us, 215 with aligned integers.  In FP32, 92 -> 80 us there, the compiler then
+// level 7 596 -> 448 us, 222 with aligned integers.  In FP32, 92 -> 80 us there, the compiler then
 // contracts the closed form's products differently, and the level's residual
 // would no longer be bit for bit that of the unsplit kernel.)
 template <class T, int DF, bool SPLIT>

@@ -3,42 +3,10 @@
 // loops over the nodes of a level inside one thread block.  Both call these
 // functions, so the two paths do the same arithmetic in the same order.
 #pragma once
-#include <type_traits>
-
 #include "hhg_aligned.cuh"
 #include "hhg_device.cuh"
 
 namespace hhg {
-
-// Closed-form stencils of regular nodes on one field: FP32 as plain sums, FP64
-// in global memory in aligned integers (hhg_aligned.cuh).  The cluster-resident
-// levels keep the FP64 sums: their phases are latency bound, with fewer warps
-// than FP64 pipes would need to be busy, and the integers spill (cube level 4
-// FP64 solve 8.50 -> 8.60 ms).
-template <class V>
-constexpr bool ALIGNED = std::is_same<V, GNb<double>>::value;
-
-template <class T, class V>
-__device__ __forceinline__ T st_nb6(const V& x) {
-  if constexpr (ALIGNED<V>)
-    return al_nb6(x);
-  else
-    return nb6v(x);
-}
-template <class T, class V>
-__device__ __forceinline__ void st_div12_all(const V& x, T out[3]) {
-  if constexpr (ALIGNED<V>)
-    al_div12_all(x, out);
-  else
-    div12_all(diff7v<T>(x), out);
-}
-template <class T, class V>
-__device__ __forceinline__ T st_div12(const V& x, int comp) {
-  if constexpr (ALIGNED<V>)
-    return al_div12(x, comp);
-  else
-    return div12(diff7v<T>(x), comp);
-}
 
 // Velocity block of the level: DF = 1 the D form (coupled 3 x 3 node blocks),
 // 0 the Laplace form, -1 read from the level (L.wt2 set in the D form).  The
@@ -78,6 +46,15 @@ __device__ __forceinline__ void node_vel_rhs(const LevelDev<T>& L, const Node& n
 // first.  Both store the same values.  u, p are neighbour views centred on
 // the node (global arrays, a shared-memory tile, or plane-pointer tables).
 
+// New velocity of a regular node from RU.
+template <class T, class V>
+__device__ __forceinline__ void vel_gs_regular(const LevelDev<T>& L, int64_t c, const V* u, T inv6nuh, T reg[3]) {
+  T nb[3];
+  st_nb6x3(u, nb);
+#pragma unroll
+  for (int d = 0; d < 3; ++d) reg[d] = (L.r[d][c] + L.nuh * nb[d]) * inv6nuh;
+}
+
 // u_d <- u_d + (RU_d - (A u_d)) / A_ii  (one node of the current colour);
 // in the D form the node's three components at once with its 3 x 3 block.
 // REG (here and below): boundary nodes are left out (the kernel updates them
@@ -97,17 +74,13 @@ __device__ __forceinline__ void node_vel_gs_v(const LevelDev<T>& L, int64_t c, c
   T reg[3];
   uint8_t fl;
   if (SPEC) {
-#pragma unroll
-    for (int d = 0; d < 3; ++d) reg[d] = (L.r[d][c] + L.nuh * st_nb6<T>(u[d])) * inv6nuh;
+    vel_gs_regular(L, c, u, inv6nuh, reg);
     fl = L.flags[c];
     if (!(fl & F_VFREE)) return;
   } else {
     fl = L.flags[c];
     if (!(fl & F_VFREE)) return;
-    if (!(fl & F_IRR)) {
-#pragma unroll
-      for (int d = 0; d < 3; ++d) reg[d] = (L.r[d][c] + L.nuh * st_nb6<T>(u[d])) * inv6nuh;
-    }
+    if (!(fl & F_IRR)) vel_gs_regular(L, c, u, inv6nuh, reg);
   }
   if (!(fl & F_IRR)) {
 #pragma unroll
@@ -168,11 +141,12 @@ __device__ __forceinline__ void vel_irr_value(const LevelDev<T>& L, const T* w, 
 template <class T, class V>
 __device__ __forceinline__ void vel_rhs_regular(const LevelDev<T>& L, int64_t c, const V* u, const V& p, T inv6nuh,
                                                 T reg[3]) {
-  T dv[3];
+  T dv[3], nb[3];
   st_div12_all<T>(p, dv);
+  st_nb6x3(u, nb);
   const T s = -L.h2 * (T)(1.0 / 12.0);
 #pragma unroll
-  for (int d = 0; d < 3; ++d) reg[d] = ((L.f[d][c] - s * dv[d]) + L.nuh * st_nb6<T>(u[d])) * inv6nuh;
+  for (int d = 0; d < 3; ++d) reg[d] = ((L.f[d][c] - s * dv[d]) + L.nuh * nb[d]) * inv6nuh;
 }
 
 // Velocity update of a boundary node (class rows) with f - B^T p formed at
@@ -268,15 +242,9 @@ __device__ __forceinline__ void node_pres_gs(const LevelDev<T>& L, const Node& n
 template <class T, class V>
 __device__ __forceinline__ T pres_regular_value(const LevelDev<T>& L, T g, const V* u, const V& p, T pc,
                                                 T omega_over_6c) {
-  const T d0 = st_div12<T>(u[0], 0);
-  const T d1 = st_div12<T>(u[1], 1);
-  const T d2 = st_div12<T>(u[2], 2);
-  const T rp = L.h2 * (T)(1.0 / 12.0) * ((d0 + d1) + d2) - g;
-  T lap;
-  if constexpr (ALIGNED<V>)
-    lap = al_lap7(p);
-  else
-    lap = (T)6 * pc - nb6v(p);
+  T d[3];
+  const T lap = st_pres(u, p, pc, d);
+  const T rp = L.h2 * (T)(1.0 / 12.0) * ((d[0] + d[1]) + d[2]) - g;
   const T cp = L.c * lap;
   return pc + omega_over_6c * (rp - cp);
 }
@@ -344,11 +312,8 @@ __device__ __forceinline__ void node_residual_v(const LevelDev<T>& L, int64_t c,
   if (REG) fl &= (uint8_t)~(F_IRR | F_SLIP);
   if constexpr (ALIGNED<V> && DF == 0) {
     if (!(fl & F_IRR)) {
-      // each field aligned once for its Laplacian and its divergence part
       T au[3], bu[3], bt[3];
-#pragma unroll
-      for (int d = 0; d < 3; ++d) au[d] = al_lap_div(u[d], d, bu + d);
-      const T cp = al_lap_div(p, -1, bt);
+      const T cp = st_residual(u, p, au, bu, bt);
       const T s = L.h2 * (T)(1.0 / 12.0);
       const bool vf = fl & F_VFREE;
 #pragma unroll
