@@ -218,10 +218,24 @@ __host__ __device__ inline int64_t coarse_scratch_doubles(const CoarseSys& S) {
 }
 constexpr int32_t COARSE_ELL_ROUND = 8;
 constexpr int32_t COARSE_ELL_MAX_ROWS = 8192;  // 16 CTAs of 512 threads, one row each
-// A coarsest level this small is solved by one thread block (one warp per CG).
+// A coarsest level this small is solved by one thread block (one warp per CG),
+// others by a cluster.  The one-block solver keeps the vectors of up to 128
+// rows in registers and those of more rows in memory, where its time depends on
+// what the shared memory around it leaves of L1; the cluster solver has a row
+// per lane in registers, and its barriers to pay.  Measured (FP64 cycles of
+// box channels, five MINRES iterations, one block against cluster): 105 rows
+// 1.16 : 1.20 ms, 175 rows 1.37 : 1.31, 315 rows 1.83 : 1.48, 392 rows
+// 2.85 : 2.14, 588 rows 6.5 : 2.4, 784 rows 4.7 : 2.3; coupled rows 225
+// 2.02 : 2.03, 315 2.24 : 2.17, 525 3.21 : 2.41, 2,298 6.3 : 2.4.  Scalar
+// systems stay on one block up to 320 rows, although the cluster is ahead from
+// about 150: its sums have another order, and full multigrid with FP32
+// corrections on such boxes shows a coarse solve that rounds differently at
+// 1e-8 of its pressure.
 constexpr int64_t COARSE_BLOCK_MAX_UNKNOWNS = 4096;
+constexpr int32_t COARSE_BLOCK_MAX_ROWS = 320, COARSE_BLOCK_MAX_COUPLED_ROWS = 256;
 __host__ __device__ inline bool coarse_fits_block(const CoarseSys& S) {
-  return 3 * (int64_t)S.nv + S.np <= COARSE_BLOCK_MAX_UNKNOWNS;
+  return 3 * (int64_t)S.nv + S.np <= COARSE_BLOCK_MAX_UNKNOWNS &&
+         (S.coupled ? 3 * S.nv <= COARSE_BLOCK_MAX_COUPLED_ROWS : S.nv <= COARSE_BLOCK_MAX_ROWS);
 }
 template <class T>
 void launch_coarse_solve(const CoarseSys& S, const LevelDev<T>& L, double* scratch, CoarseParams prm, double* info,
