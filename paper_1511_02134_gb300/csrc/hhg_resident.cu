@@ -532,7 +532,15 @@ __global__ void __launch_bounds__(RT) k_resident(const __grid_constant__ Residen
 }  // namespace
 
 // Lays out the shared memory for per-level CTA counts nbq (cluster size the
-// largest of them); returns the bytes per CTA.
+// largest of them); returns the bytes per CTA.  The coarse solve's memory
+// (3.8 KB, or 16 KB where the cluster solves the coarsest level) lies ahead of
+// the levels, and a level that would fit only without it is launched per
+// colour: so near the limit that is the faster side, since the launches spread
+// its nodes over all SMs and leave the coarse solve its L1.  Measured per
+// cycle, such a level held (the coarse solve's memory laid over the residuals)
+// against launched: FP64 channel of 9 x 4 x 4 cubes 2.71 : 2.30 ms, 11 x 4 x 4
+// 2.83 : 2.35; FP32 12 x 4 x 4 2.06 : 1.91, 16 x 3 x 4 1.88 : 1.74; box of
+// 5 x 2 x 2 at level 5 (level 3 held or not) 1.80 : 1.75.
 template <class T>
 uint64_t layout_resident(ResidentCycle<T>& S) {
   unsigned nb = 1;
