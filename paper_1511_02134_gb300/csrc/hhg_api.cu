@@ -1076,7 +1076,7 @@ int hhg_create_mesh(const double* V, int64_t nv, const int32_t* T, int64_t nt, c
       // boundary block's extra load (its list entry) costs more there than the
       // divergence it avoids: FP32 Uzawa step, level 5 27.5 -> 31.3 us, level 6
       // 39.2 -> 44.8 us, level 7 121 -> 103 us; FP64 level 5 71 -> 50 us.
-      L.split = H.nirr > 0 && 2 * H.nirr < H.n_pres && (sizeof(L.nuh) == 8 || !L.spec);
+      L.split = H.nirr > 0 && 2 * H.nirr < H.n_pres && (sizeof(L.nuh) == 8 || !L.spec) && boundary_grids_fit(L);
     };
     bind_boundary(H.d64);
     bind_boundary(H.d32);

@@ -45,6 +45,13 @@ template <class T>
 dim3 full_grid(const LevelDev<T>& L) {
   return dim3((L.nx + FX - 1) / FX, (L.ny + FY - 1) / FY, L.nz);
 }
+// Boundary nodes of the residual, in the first `rows` planes of its grid.
+template <class T>
+BoundaryNodes residual_boundary(const LevelView<T>& L) {
+  const dim3 grid = full_grid(L);
+  const int64_t n = L.bnd_at[1][4], plane = (int64_t)grid.x * grid.y * (FX * FY);
+  return BoundaryNodes{L.bnd[1], (int)n, (int)((n + plane - 1) / plane)};
+}
 
 // Whether the level's colour kernels use the speculative node form
 // (hhg_node_ops.cuh); set per level by the host (hhg_options.spec_max_nodes).
@@ -1435,6 +1442,14 @@ void launch_pres_colour(const LevelDev<T>& L, int colour, cudaStream_t s) {
   launch_k(k_pres_colour<T>, colour_grid(L, 0), colour_block(L), s, L, colour, w);
 }
 template <class T>
+bool boundary_grids_fit(const LevelView<T>& L) {
+  constexpr int64_t MOST = 65535;
+  for (int kind = 0; kind < 2; ++kind)
+    for (int c = 0; c < 4; ++c)
+      if (colour_grid(L, boundary_nodes(L, kind, c, true).rows).y > MOST) return false;
+  return L.nz + (int64_t)residual_boundary(L).rows <= MOST;
+}
+template <class T>
 void launch_residual(const LevelView<T>& L, cudaStream_t s) {
   if (!L.wt2 && L.quad) {
     const int npos = L.nx / 4 + 1;  // quads cover padded x = 0 .. 4 npos - 1 >= nx
@@ -1446,8 +1461,7 @@ void launch_residual(const LevelView<T>& L, cudaStream_t s) {
   const bool split = SP && L.split;
   BoundaryNodes B{nullptr, 0, 0};
   if (split) {
-    const int64_t n = L.bnd_at[1][4], plane = (int64_t)grid.x * grid.y * (FX * FY);
-    B = BoundaryNodes{L.bnd[1], (int)n, (int)((n + plane - 1) / plane)};
+    B = residual_boundary(L);
     grid.z += B.rows;
   }
   auto go = [&](auto kernel) { launch_k(kernel, grid, dim3(FX, FY), s, L, B); };
@@ -1604,6 +1618,7 @@ void launch_cast_field(const double* src, float* dst, int64_t n, cudaStream_t s)
   template void launch_pres_colour_rhs<T>(const LevelView<T>&, int, cudaStream_t);                       \
   template void launch_vel_pres_colour0<T>(const LevelView<T>&, bool, cudaStream_t);                      \
   template void launch_pres_colour<T>(const LevelDev<T>&, int, cudaStream_t);                           \
+  template bool boundary_grids_fit<T>(const LevelView<T>&);                                              \
   template void launch_residual<T>(const LevelView<T>&, cudaStream_t);                                   \
   template void launch_restrict<T>(const LevelDev<T>&, const LevelDev<T>&, cudaStream_t);               \
   template void launch_prolong_add<T>(const LevelDev<T>&, const LevelDev<T>&, cudaStream_t);            \

@@ -74,6 +74,10 @@ void prepare_fused();
 // (hhg_node_ops.cuh).  Measured on GB300: a level-5 FP32 Uzawa step 37.9 ->
 // 28.2 us, level 6 60 -> 49 us, while level 7 went 170 -> 191 us.
 constexpr int64_t SPEC_MAX_NODES = 1 << 20;
+// Whether the grids of the colour and residual kernels hold the level's planes
+// and its boundary blocks (65,535 blocks along y and z: lattices of more than
+// about 58,000 planes do not).
+template <class T> bool boundary_grids_fit(const LevelView<T>& L);
 // Residual (RU, RP) = (F, G) - K (U, P); zero on nodes without unknowns.
 template <class T> void launch_residual(const LevelView<T>& L, cudaStream_t s);
 
