@@ -118,7 +118,7 @@ __device__ __noinline__ int cg_team_regs(const Ctx& C, const double* b, double* 
   int its = 0;
   if (live) team_publish(T, rv * rv, mine, group);
   double res[2 * NSYS];
-  team_finish<NSYS, 2>(T, groups, res, [&](int, double tot, double* out) {
+  team_finish<NSYS, 2>(T, groups, res, [&](double tot, double* out) {
     rr = tot;
     stop = rtol * rtol * tot;
     run = !(rr <= stop || rr == 0.0);
@@ -157,7 +157,7 @@ __device__ __noinline__ int cg_team_regs(const Ctx& C, const double* b, double* 
       if (!on) qv = 0.0;
       team_publish(T, dv * qv, mine, group);
     }
-    team_finish<NSYS, 2>(T, groups, res, [&](int, double tot, double* out) {
+    team_finish<NSYS, 2>(T, groups, res, [&](double tot, double* out) {
       if (run && tot == 0.0) run = false;
       out[0] = run ? 1.0 : 0.0;
       out[1] = run ? rr / tot : 0.0;
@@ -169,7 +169,7 @@ __device__ __noinline__ int cg_team_regs(const Ctx& C, const double* b, double* 
       team_publish(T, rv * rv, mine, group);
       xv = fma(alpha, dv, xv);
     }
-    team_finish<NSYS, 2>(T, groups, res, [&](int, double tot, double* out) {
+    team_finish<NSYS, 2>(T, groups, res, [&](double tot, double* out) {
       out[0] = out[1] = 0.0;
       if (run) {
         out[1] = tot / rr;
@@ -186,7 +186,7 @@ __device__ __noinline__ int cg_team_regs(const Ctx& C, const double* b, double* 
     T.sync();
   }
   if (on) x[idx] = xv;
-  team_finish<NSYS, 1>(T, 0, res, [&](int, double, double* out) { out[0] = (double)its; });
+  team_finish<NSYS, 1>(T, 0, res, [&](double, double* out) { out[0] = (double)its; });
   double n = 0.0;
 #pragma unroll
   for (int s = 0; s < NSYS; ++s) n += res[s];
@@ -231,7 +231,7 @@ __device__ __noinline__ int cg_team_mem(const Ctx& C, const double* b, double* x
   int its = 0;
   publish(acc);
   double res[2 * NSYS];
-  team_finish<NSYS, 2>(T, groups, res, [&](int, double tot, double* out) {
+  team_finish<NSYS, 2>(T, groups, res, [&](double tot, double* out) {
     rr = tot;
     stop = rtol * rtol * tot;
     run = !(rr <= stop || rr == 0.0);
@@ -254,7 +254,7 @@ __device__ __noinline__ int cg_team_mem(const Ctx& C, const double* b, double* x
       }
     }
     publish(acc);
-    team_finish<NSYS, 2>(T, groups, res, [&](int, double tot, double* out) {
+    team_finish<NSYS, 2>(T, groups, res, [&](double tot, double* out) {
       if (run && tot == 0.0) run = false;
       out[0] = run ? 1.0 : 0.0;
       out[1] = run ? rr / tot : 0.0;
@@ -274,7 +274,7 @@ __device__ __noinline__ int cg_team_mem(const Ctx& C, const double* b, double* x
         }
     }
     publish(acc);
-    team_finish<NSYS, 2>(T, groups, res, [&](int, double tot, double* out) {
+    team_finish<NSYS, 2>(T, groups, res, [&](double tot, double* out) {
       out[0] = out[1] = 0.0;
       if (run) {
         out[1] = tot / rr;
@@ -292,7 +292,7 @@ __device__ __noinline__ int cg_team_mem(const Ctx& C, const double* b, double* x
       }
     T.sync();
   }
-  team_finish<NSYS, 1>(T, 0, res, [&](int, double, double* out) { out[0] = (double)its; });
+  team_finish<NSYS, 1>(T, 0, res, [&](double, double* out) { out[0] = (double)its; });
   double n = 0.0;
 #pragma unroll
   for (int s = 0; s < NSYS; ++s) n += res[s];
@@ -619,7 +619,7 @@ __device__ __noinline__ void minres_team(const Team& tm, const CoarseSys& S, con
   // sum (team_finish) and published
   double gamma;
   team_reduce1<1>(C.T, dot_part(C, zz[iz], vv[iv]), n, &gamma,
-                  [](int, double tot, double* out) { out[0] = sqrt(fmax(tot, 0.0)); });
+                  [](double tot, double* out) { out[0] = sqrt(fmax(tot, 0.0)); });
   int its = 0;
   double rel = 0.0;
   if (gamma > 0.0) {
@@ -631,7 +631,7 @@ __device__ __noinline__ void minres_team(const Team& tm, const CoarseSys& S, con
       tm.sync();
       applyK(C, zz[iz], Kz);
       double r[3];
-      team_reduce1<3>(C.T, dot_part(C, Kz, zz[iz]), n, r, [=](int, double tot, double* out) {
+      team_reduce1<3>(C.T, dot_part(C, Kz, zz[iz]), n, r, [=](double tot, double* out) {
         out[0] = tot;
         out[1] = tot / gamma;
         out[2] = gamma / gamma_prev;
@@ -642,7 +642,7 @@ __device__ __noinline__ void minres_team(const Team& tm, const CoarseSys& S, con
       tm.sync();
       cg_total += precond(C, vv[iv_next], zz[iz_next], cg, prm.cg_max, prm.cg_rtol);
       double g[6];
-      team_reduce1<6>(C.T, dot_part(C, zz[iz_next], vv[iv_next]), n, g, [=](int, double tot, double* out) {
+      team_reduce1<6>(C.T, dot_part(C, zz[iz_next], vv[iv_next]), n, g, [=](double tot, double* out) {
             const double gamma_next = sqrt(fmax(tot, 0.0));
             const double a0 = fma(cc, delta, -(c_prev * ss * gamma));
             const double a1 = sqrt(fma(a0, a0, gamma_next * gamma_next));

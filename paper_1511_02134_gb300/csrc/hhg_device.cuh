@@ -136,11 +136,6 @@ __device__ __forceinline__ auto nb6v(const V& x) {
   return ((x(-1, 0, 0) + x(1, 0, 0)) + (x(0, -1, 0) + x(0, 1, 0))) + (x(0, 0, -1) + x(0, 0, 1));
 }
 
-template <class T>
-__device__ __forceinline__ T nb6(const T* x, const Node& n, int64_t px, int64_t pxy) {
-  return nb6v(gnb(x, n, px, pxy));
-}
-
 // Antisymmetric differences x(c+o) - x(c-o) over the 7 Kuhn directions.
 template <class T>
 struct Diff7 {

@@ -1,7 +1,10 @@
 // Per-node bodies of the smoother, residual and transfer steps (Sec. 3.3-3.5).
 // The grid kernels run one node per thread; the fused coarse-levels kernel
 // loops over the nodes of a level inside one thread block.  Both call these
-// functions, so the two paths do the same arithmetic in the same order.
+// functions and evaluate the same expressions; the FP64 sums of regular nodes
+// are formed in aligned integers on global memory and as plain operations in
+// the cluster-resident levels and in the fused kernel's residual (the st_*
+// functions of hhg_aligned.cuh), so there the two paths differ by rounding.
 #pragma once
 #include "hhg_aligned.cuh"
 #include "hhg_device.cuh"

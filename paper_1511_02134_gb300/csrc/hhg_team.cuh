@@ -81,7 +81,7 @@ __device__ __forceinline__ void team_publish(const Team& T, double x, int w, int
 
 // Totals of the W sums just published (groups 0 .. ngroups - 1 of each).
 // Warp w < W of every CTA is the handler of sum w: it evaluates
-// fin(w, total, out) in all its lanes (out: W_OUT doubles published to the
+// fin(total, out) in all its lanes (out: W_OUT doubles published to the
 // CTA), so that the scalar recurrences of a Krylov step run in one warp per
 // CTA.  On GB300 an FP64 instruction occupies a quarter of an SM for 64
 // cycles per warp: evaluated by every thread, the partials of sixteen CTAs,
@@ -118,7 +118,7 @@ __device__ __forceinline__ void team_finish(const Team& T, int ngroups, double* 
     double tot = __shfl_sync(0xffffffffu, run, 0);
     for (int c = 1; c * per < ngroups; ++c) tot += __shfl_sync(0xffffffffu, run, c);
     double out[W_OUT];
-    fin(warp, tot, out);
+    fin(tot, out);
     if (every) {
 #pragma unroll
       for (int e = 0; e < W_OUT; ++e) vals[e] = out[e];
