@@ -11,8 +11,8 @@
 // in place of 64 per addition (the divergence sums of one field take 16
 // operations per component).
 // Measured (cube level 7, with boundary nodes in blocks of their own): Uzawa
-// step 567 -> 354 us, its pressure sweep 275 -> 144 us, residual 448 -> 222 us;
-// level 8 Uzawa step 4.75 (unsplit) -> 2.63 ms.
+// step 567 -> 347 us, its pressure sweep 275 -> 134 us, residual 448 -> 223 us;
+// level 8 Uzawa step 4.75 (unsplit) -> 2.56 ms.
 //
 // Accuracy (u = 2^-53): where every value of a stencil that is not zero has an
 // exponent within G of the largest, no bit is cut off: the sum is exact,
@@ -23,13 +23,13 @@
 // values then count in full; so a stencil with cut values is summed in
 // integers only where the largest pair (the difference of two opposite
 // neighbours in a divergence, their sum in a Laplacian, or the centre) is
-// close to the largest value.  The sum is then off by at most 1.5 u (six
-// neighbours), 3 u (Laplacian) or 4.5 u (divergence) of that pair and one
-// rounding, where the FP64 operations may round that pair and each of the up
-// to nine sums it enters.  Over random stencils of one and of many magnitudes,
-// with cancelling pairs and zero crossings, the rms error of the stencils with
-// cut values is 0.45 to 0.99 of theirs.  (Two pairs that cancel each other are
-// not looked for.)
+// within 2^-K of the largest value (AlSums::note).  The sum is then off by at
+// most 3 u (six neighbours), 6 u (Laplacian) or 9 u (divergence) of that pair
+// and one rounding, where the FP64 operations may round that pair and each of
+// the up to nine sums it enters.  Over ten kinds of random stencils (one and
+// many magnitudes, equal, close and opposite pairs, ramps) the rms error of
+// those with cut values is 0.45 to 1.0 of the FP64 operations'.  (Two pairs
+// that cancel each other are not looked for.)
 //
 // All other stencils take the FP64 operations: those without such a pair, and
 // those whose largest value is not finite, or so large that the sum could
@@ -38,8 +38,8 @@
 // (al_fp64_*), which reads the values again: kept in registers beside their
 // integers they would cost all nodes.
 // Measured (cube level 7, a solve's last state): FP64 wherever a value is cut
-// off 65.2 ms per solve, pairs within the largest value's exponent or one
-// below 59.9, two below (here) 57.6, every stencil in integers 56.8.
+// off 65.2 ms per solve, K smaller by two 59.9, by one 57.7, as here 57.3,
+// every stencil in integers 56.8.
 #pragma once
 #include <type_traits>
 
@@ -149,16 +149,15 @@ __device__ __forceinline__ int64_t al_sum6(const int64_t* i, int32_t& pair) {
 }
 
 // Stencil sums of one node in aligned integers.  Each sum has a bit, set in bad
-// if it has to be formed in FP64.  (Once a stencil is out of range the
-// remaining ones are left to FP64 as well: without that branch between them
-// the compiler loads all fields ahead and keeps half as many warps.)
+// if it has to be formed in FP64.  (The divergences leave a stencil that is
+// out of range at once: that branch keeps the compiler from loading all fields
+// ahead, which costs half the warps, and leaves it the next field's loads
+// beside this one's conversions.)
 struct AlSums {
   unsigned bad = 0;
-  bool out = false;
 
   template <int K, int G>
   __device__ __forceinline__ void note(const AlTop<G>& t, int32_t pair, unsigned bit) {
-    out |= !t.in;
     if (!t.holds<K>(pair)) bad |= bit;
   }
 
@@ -172,17 +171,13 @@ struct AlSums {
     for (int n = 0; n < 6; ++n) i[n] = al_int<G>(v[n], t.top);
     int32_t pair;
     const int64_t s = al_sum6(i, pair);
-    note<4>(t, pair, bit);
+    note<5>(t, pair, bit);
     return al_value<G>(s, t.top);
   }
 
   // 6 x(c) minus the six axis neighbours (12 2^59 < 2^63).
   __device__ __forceinline__ double lap7(const GNb<double>& x, double xc, unsigned bit) {
     constexpr int G = 6;
-    if (out) {
-      bad |= bit;
-      return 0.0;
-    }
     const double v[7] = {x(-1, 0, 0), x(1, 0, 0), x(0, -1, 0), x(0, 1, 0), x(0, 0, -1), x(0, 0, 1), xc};
     const AlTop<G> t(v);
     int64_t i[6];
@@ -190,7 +185,7 @@ struct AlSums {
     for (int n = 0; n < 6; ++n) i[n] = al_int<G>(v[n], t.top);
     int32_t pair;
     const int64_t nb = al_sum6(i, pair), c = al_int<G>(xc, t.top);
-    note<3>(t, max(pair, al_pair(c)), bit);
+    note<4>(t, max(pair, al_pair(c)), bit);
     return al_value<G>(6 * c - nb, t.top);
   }
 
@@ -200,7 +195,7 @@ struct AlSums {
   static constexpr int DG = 5;
   __device__ __forceinline__ void div12_in(const AlTop<DG>& t, const int64_t (&i)[14], int comp, double* div, unsigned bit) {
     const Diff7<int64_t> d = al_diff7<int64_t>(i);
-    note<2>(t, al_pair14(d), bit);
+    note<3>(t, al_pair14(d), bit);
     if (comp < 0) {
       int64_t o[3];
       div12_all(d, o);
@@ -211,13 +206,13 @@ struct AlSums {
     }
   }
   __device__ __forceinline__ void div12_of(const GNb<double>& x, int comp, double* div, unsigned bit) {
-    if (out) {
-      bad |= bit;
-      return;
-    }
     double v[14];
     al_load14(x, v);
     const AlTop<DG> t(v);
+    if (!t.in) {
+      bad |= bit;
+      return;
+    }
     int64_t i[14];
 #pragma unroll
     for (int n = 0; n < 14; ++n) i[n] = al_int<DG>(v[n], t.top);
@@ -232,15 +227,15 @@ struct AlSums {
   // the Laplacian's, 16 bit the divergence's.
   __device__ __forceinline__ double lap_div(const GNb<double>& x, int comp, double* div, unsigned bit) {
     constexpr int G = DG;
-    if (out) {
-      bad |= 17 * bit;
-      return 0.0;
-    }
     double v[14];
     al_load14(x, v);
     const double l[7] = {v[0], v[1], v[2], v[3], v[4], v[5], x(0, 0, 0)};
     const AlTop<G> t(v);
     AlTop<G> tl(l);
+    if (!t.in || !tl.in) {
+      bad |= 17 * bit;
+      return 0.0;
+    }
     const uint32_t below = (t.top >> 21) - (tl.top >> 21);  // wraps where the centre is the largest
     int64_t i[14];
 #pragma unroll
@@ -255,7 +250,7 @@ struct AlSums {
     }
     int32_t pair;
     const int64_t nb = al_sum6(i, pair), c = al_int<G>(l[6], tl.top);
-    note<2>(tl, max(pair, al_pair(c)), bit);
+    note<3>(tl, max(pair, al_pair(c)), bit);
     return al_value<G>(6 * c - nb, tl.top);
   }
 };

@@ -87,8 +87,9 @@ struct BoundaryNodes {
 // (griddepcontrol.wait returns at once when there is no such grid), then lets
 // its own dependent grid be scheduled; no kernel touches device memory before
 // the wait.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_enter() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  pdl_wait();
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 

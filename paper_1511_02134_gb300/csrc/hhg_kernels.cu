@@ -32,7 +32,7 @@ dim3 colour_grid(const LevelDev<T>& L, int by) {
 // lattice order the two ends of a row put a boundary node into 45 % of the
 // warps of a level-7 pressure colour, and each such warp walked the class
 // rows (110 more loads, 65 multiply-adds) beside the closed form.  Measured:
-// cube level 7 pressure sweep, FP32 62.2 -> 46.1 us, FP64 428 -> 275 us (144
+// cube level 7 pressure sweep, FP32 62.2 -> 46.1 us, FP64 428 -> 275 us (134
 // with the closed form in aligned integers, hhg_aligned.cuh).
 template <class T>
 BoundaryNodes boundary_nodes(const LevelView<T>& L, int kind, int colour, bool split) {
@@ -136,6 +136,19 @@ __global__ void __launch_bounds__(CB * 4) k_vel_colour_rhs(LevelDev<T> L, int co
   node_vel_gs_rhs<SPEC, T, DF, SPLIT>(L, node_at(L.px, L.pxy, i, j, k), inv6nuh);
 }
 
+// Entry of the kernels with a pressure update.  In FP64 the next grid is let in
+// as blocks end, not at once: five blocks per SM (80 to 96 registers) hold all
+// of a level-6 colour, early blocks of the next one then fill the SMs that have
+// room and leave it unevenly spread.  Measured: FP64 pressure sweep, cube level
+// 6 46 -> 29 us, level 5 23.0 -> 21.4; Uzawa step 78 -> 68 and 45 -> 43 us.
+template <class T>
+__device__ __forceinline__ void pres_enter() {
+  if (sizeof(T) == 8)
+    pdl_wait();
+  else
+    pdl_enter();
+}
+
 // The last velocity colour of a step (backward colour 0) and the first
 // pressure colour in one launch.  A pressure node of colour 0 reads the
 // velocity of its neighbours, which are of the other colours and final
@@ -156,7 +169,7 @@ __device__ __forceinline__ void vel_pres_node(const LevelDev<T>& L, const Node& 
 
 template <class T, bool RU, bool SPEC, int DF, bool SPLIT>
 __global__ void __launch_bounds__(CB * 4) k_vel_pres_colour0(LevelDev<T> L, T inv6nuh, T omega_over_6c, BoundaryNodes B) {
-  pdl_enter();
+  pres_enter<T>();
   if (SPLIT && (int)blockIdx.y < B.rows) {
     Node n;
     if (boundary_node(L, B, colour_thread(), n))
@@ -170,7 +183,7 @@ __global__ void __launch_bounds__(CB * 4) k_vel_pres_colour0(LevelDev<T> L, T in
 
 template <class T, bool SPEC, bool SPLIT>
 __global__ void __launch_bounds__(CB * 4) k_pres_colour_rhs(LevelDev<T> L, int colour, T omega_over_6c, BoundaryNodes B) {
-  pdl_enter();
+  pres_enter<T>();
   if (SPLIT && (int)blockIdx.y < B.rows) {
     Node n;
     if (boundary_node(L, B, colour_thread(), n)) node_pres_gs_rhs<false>(L, n, omega_over_6c);
@@ -317,7 +330,7 @@ __global__ void __launch_bounds__(CB * 4) k_pres_colour(LevelDev<T> L, int colou
 }
 
 // SPLIT: boundary nodes in the first B.rows planes of blocks (FP64 only: cube
-// level 7 596 -> 448 us, 222 with aligned integers.  In FP32, 92 -> 80 us there, the compiler then
+// level 7 596 -> 448 us, 223 with aligned integers.  In FP32, 92 -> 80 us there, the compiler then
 // contracts the closed form's products differently, and the level's residual
 // would no longer be bit for bit that of the unsplit kernel.)
 template <class T, int DF, bool SPLIT>
