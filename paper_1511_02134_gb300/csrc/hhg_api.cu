@@ -1036,6 +1036,11 @@ int hhg_create_mesh(const double* V, int64_t nv, const int32_t* T, int64_t nt, c
             if (f & F_VFREE) by_colour[0][(i + j + k) & 3].push_back(e);
           }
         }
+    // on affine lattices every node takes class rows: nothing to keep apart
+    const bool apart = 2 * (int64_t)(by_colour[1][0].size() + by_colour[1][1].size() + by_colour[1][2].size() +
+                                     by_colour[1][3].size()) < H.n_pres;
+    if (!apart)
+      for (std::vector<int64_t>& v : by_colour[0]) v = {};
     std::vector<int64_t> virr;
     for (int kind = 0; kind < 2; ++kind)
       for (int c = 0; c < 4; ++c) {
@@ -1071,12 +1076,11 @@ int hhg_create_mesh(const double* V, int64_t nv, const int32_t* T, int64_t nt, c
       L.bnd[1] = H.d_irr;
       for (int kind = 0; kind < 2; ++kind)
         for (int c = 0; c < 5; ++c) L.bnd_at[kind][c] = H.bnd_at[kind][c];
-      // on affine lattices every node takes class rows: nothing to keep apart.
       // The FP32 levels of the speculative form are latency bound, and a
       // boundary block's extra load (its list entry) costs more there than the
       // divergence it avoids: FP32 Uzawa step, level 5 27.5 -> 31.3 us, level 6
       // 39.2 -> 44.8 us, level 7 121 -> 103 us; FP64 level 5 71 -> 50 us.
-      L.split = H.nirr > 0 && 2 * H.nirr < H.n_pres && (sizeof(L.nuh) == 8 || !L.spec) && boundary_grids_fit(L);
+      L.split = H.nirr > 0 && apart && (sizeof(L.nuh) == 8 || !L.spec) && boundary_grids_fit(L);
     };
     bind_boundary(H.d64);
     bind_boundary(H.d32);
